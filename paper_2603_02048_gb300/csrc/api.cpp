@@ -105,6 +105,12 @@ cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 // 64-bit linear offsets.
 constexpr int kMaxAxis = 1 << 14;
 
+// Voxels of the grid with its one-voxel halo, every axis padded to even. A
+// ZPAIR volume pads its rows further, which adds at most three quarters.
+size_t stored_voxels(const hh_grid* g) {
+    return static_cast<size_t>((g->nx + 3) / 2) * ((g->ny + 3) / 2) * ((g->nz + 3) / 2) * 8;
+}
+
 hh_status check_grid(const hh_grid* g, bool need_h) {
     if (!g) return fail(HH_ERR_INVALID_ARG, "grid is NULL");
     if (g->nx < 2 || g->ny < 2 || g->nz < 2 || g->nx > kMaxAxis || g->ny > kMaxAxis ||
@@ -113,8 +119,7 @@ hh_status check_grid(const hh_grid* g, bool need_h) {
                     g->ny, g->nz, kMaxAxis);
     if (g->storage != HH_STORE_FP32 && g->storage != HH_STORE_FP16_SCALED)
         return fail(HH_ERR_INVALID_ARG, "unknown storage %d", g->storage);
-    if (static_cast<size_t>(brick2_count(g->nx)) * brick2_count(g->ny) * brick2_count(g->nz) * 8 >
-        (size_t(1) << 31))
+    if (stored_voxels(g) > (size_t(1) << 31))
         return fail(HH_ERR_INVALID_ARG, "grid %d x %d x %d: more than 2^31 stored voxels", g->nx,
                     g->ny, g->nz);
     if (need_h && !(g->h_kernel > 0.0f && std::isfinite(g->h_kernel)))
@@ -144,27 +149,28 @@ hh_status new_volume(const hh_grid* g, hh_volume* out) {
     v->nz = g->nz;
     v->storage = g->storage;
     v->h_kernel = g->h_kernel;
-    v->layout = HH_LAYOUT_BRICK2;
-    v->bx = brick2_count(g->nx);
-    v->bxy = v->bx * brick2_count(g->ny);
-    const size_t padded = static_cast<size_t>(v->bxy) * brick2_count(g->nz) * 8;
-    v->bytes = padded * (g->storage == HH_STORE_FP32 ? 16 : 8);
-    v->bz = brick2_count(g->nz);
-    v->mask_words = (padded + 31) / 32;  // one bit per element (8 per brick, a byte)
-    // the free-corner mask and its build scratch (a word per stored column
-    // and 16-slice z run, rows padded to 4 columns) follow the data in the
-    // same allocation (the data's size is a multiple of 64 bytes, so the mask
-    // is aligned); all of it starts zero: even-padding voxels read as 0, and
-    // no element is marked free before the first build
-    const size_t colbytes = static_cast<size_t>((g->nx + 2 + 3) & ~3) * (g->ny + 2) *
-                            ((g->nz + 15) / 16) * sizeof(uint32_t);
-    const size_t total = v->bytes + v->mask_words * sizeof(unsigned) + colbytes;
+    v->layout = HH_LAYOUT_ZPAIR;
+    v->row = zpair_row(g->nx);
+    v->pair = zpair_pair(g->nx, g->ny);
+    const size_t voxel_bytes = g->storage == HH_STORE_FP32 ? 16 : 8;
+    v->bytes = stored_voxels(g) * voxel_bytes;
+    // the free-corner mask, its build scratch (a bit per element and voxel)
+    // and the sparse flag follow the data in the same allocation; all of it
+    // starts zero: no element is marked free before the first build
+    const size_t pairs = (static_cast<size_t>(g->nz) + 3) / 2;
+    const size_t elements = static_cast<size_t>(v->pair) * pairs;
+    const size_t mask_words = (elements + 31) / 32;
+    v->nz_words = (static_cast<unsigned>(g->nx) + 2u + 31u) / 32u;
+    const size_t nz_total = 2 * pairs * (static_cast<size_t>(g->ny) + 3) * v->nz_words;
+    v->mask_off = (elements * voxel_bytes + 255) & ~size_t(255);
+    const size_t total = v->mask_off + (mask_words + nz_total + 1) * sizeof(unsigned);
     cudaGetDevice(&v->device);
     cudaError_t e = dev_alloc(&v->data, total);
     if (e == cudaSuccess) e = cudaMemset(v->data, 0, total);
     if (e == cudaSuccess) {
-        v->free_dev = reinterpret_cast<unsigned*>(static_cast<char*>(v->data) + v->bytes);
-        v->colbits_dev = reinterpret_cast<uint32_t*>(v->free_dev + v->mask_words);
+        v->free_dev = reinterpret_cast<unsigned*>(static_cast<char*>(v->data) + v->mask_off);
+        v->nz_dev = v->free_dev + mask_words;
+        v->sparse_dev = v->nz_dev + nz_total;
     }
     if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void**>(&v->scales_dev), 2 * sizeof(float));
     if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void**>(&v->max_dev), 2 * sizeof(unsigned));

@@ -8,46 +8,20 @@
 //         reduces the maxima, pass 2 recomputes the differences and quantises
 //         with exact multiplications by 1 / s; rho is read twice, nothing else
 //         stored).
-// Threads map to (x, y) columns, x fastest (a warp is 32 consecutive
-// columns), and walk 16 z slices each, so every load of rho is coalesced, the
-// z neighbours come from registers and the x/y neighbours from L1.
-// The packed volume is written in the volume's layout (BRICK2 with its halo
-// of edge copies for volumes the march reads, LINEAR for the allocation-free
-// build's caller buffer); in BRICK2 the x-pairs of a warp land in whole
-// 32-byte sectors. The volume stores are marked evict-first (st.global.cs):
-// the volume outgrows L2 anyway, and this keeps the density, which the
-// kernel is still reading, resident in L2 instead.
-// BRICK2 builds also leave the volume's free-corner mask (the march skips the
+// The packed volume is written in the volume's layout (ZPAIR with its halo of
+// edge copies for volumes the march reads, LINEAR for the allocation-free
+// build's caller buffer). The ZPAIR FP32 stores are marked evict-first: the
+// volume outgrows L2 anyway, and this keeps the density, which the kernel is
+// still reading, resident in L2 instead.
+// ZPAIR builds also leave the volume's free-corner mask (the march skips the
 // eight loads of a sample whose corners are all zero): the store pass records
-// per column and run which slices hold a nonzero stored voxel (a 32-bit word,
-// no atomics), and free_mask_kernel turns those into one bit per stored
-// voxel, set when the eight voxels of the cell it is the first corner of are
-// all zero. The store passes walk their runs unrolled by 2, not 4: with the
-// column's bits to carry, 4 spilled and was slower.
+// which voxels are nonzero (ballots, no atomics), and free_mask_kernel turns
+// those into one bit per element, set when the eight voxels of the cell it is
+// the first corner of are all zero.
 #include "hh_internal.h"
 
 namespace hh {
 namespace {
-
-struct Cell {
-    float dn, gx, gy, gz;
-};
-
-struct OutLayout {
-    int layout;
-    unsigned bx, bxy;
-    uint32_t* colbits;    // BRICK2: per stored (padded) column and z run, the slices
-                          // where it stored a nonzero voxel (null: none); rows of
-                          // `pitch` columns
-    int pitch;
-};
-
-// Element of grid voxel (i, j, k) in the output layout (BRICK2: halo offset).
-__device__ __forceinline__ size_t out_index(const OutLayout& L, int i, int j, int k, int nx,
-                                            int ny) {
-    if (L.layout == HH_LAYOUT_BRICK2) return brick2_offset(i + 1, j + 1, k + 1, L.bx, L.bxy);
-    return (static_cast<size_t>(k) * ny + j) * nx + i;
-}
 
 // Scale of a channel group from the bit pattern of its maximum |value| m:
 // the smallest power of two s with m / s <= HH_FP16_CODE_MAX (the largest code
@@ -62,110 +36,201 @@ __device__ __forceinline__ float scale_of(unsigned bits) {
     return __uint_as_float(b);
 }
 
-// Column variant: each thread owns one (i, j) column and walks a run of
-// FIELD_ZRUN slices, keeping rho at k-1, k, k+1 in registers, so rho is read
-// from memory about once per voxel plus the four x/y neighbours (L1 hits).
-#define FIELD_ZRUN 16
+// 32 bytes to an aligned address in one store, evict-first in L2.
+__device__ __forceinline__ void store32(void* p, uint4 a, uint4 b) {
+    asm volatile("st.global.L2::evict_first.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z),
+                 "r"(b.w)
+                 : "memory");
+}
 
-// 8 resident blocks of 256 threads for every mode (32 registers); the FP16
-// store pass with 5 (48 registers) was 6-8 % slower, and with 6 or 7 it
-// spilled more, not less.
-template <int MODE>  // 0: FP32 store, 1: FP16 max pass, 2: FP16 store
-__global__ void __launch_bounds__(256, 8) field_column_kernel(const float* __restrict__ rho, int nx,
-                                                           int ny, int nz, float K, OutLayout L,
-                                                           void* __restrict__ out,
-                                                           unsigned* __restrict__ max_bits,
-                                                           float* __restrict__ scales) {
-    // Threads cover the stored (x, y) columns (I, J), x fastest, 256 per block
-    // (a warp is 32 consecutive columns, wrapping across rows). With the
-    // BRICK2 halo (h = 1, stores only) every stored column, halo included, is
-    // written by its own thread with the values of grid column (clamp(I - 1),
-    // clamp(J - 1)), the halo's copy of the nearest edge column; the z halo
-    // slices repeat the first and last grid slice.
-    const int h = (MODE != 1 && L.layout == HH_LAYOUT_BRICK2) ? 1 : 0;
-    const int W = nx + 2 * h, Hh = ny + 2 * h;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int J = t / W, I = t - J * W;
-    const int k0 = blockIdx.y * FIELD_ZRUN;
-    const int k1 = min(k0 + FIELD_ZRUN, nz);
+// One voxel's {dn, gx, gy, gz}, as stored: FP32, or halves of value / s (the
+// nearest half; the products are exact as s is a power of two).
+struct Voxel {
+    float dn, gx, gy, gz;
+};
+__device__ __forceinline__ uint4 pack32(const Voxel& v) {
+    return make_uint4(__float_as_uint(v.dn), __float_as_uint(v.gx), __float_as_uint(v.gy),
+                      __float_as_uint(v.gz));
+}
+__device__ __forceinline__ uint2 pack16(const Voxel& v, float rs_n, float rs_g) {
+    const __half2 lo = __floats2half2_rn(v.dn * rs_n, v.gx * rs_g);
+    const __half2 hi = __floats2half2_rn(v.gy * rs_g, v.gz * rs_g);
+    return make_uint2(*reinterpret_cast<const unsigned*>(&lo),
+                      *reinterpret_cast<const unsigned*>(&hi));
+}
+
+// A thread owns voxel column I of a pair of rows J = 2 jj, 2 jj + 1 and walks
+// `run` pairs of slices K = 2 kk, 2 kk + 1: four voxels an iteration. A row's two
+// are consecutive in the ZPAIR layout, so a warp stores 1 KiB (FP32) or 512 B
+// (FP16) in one piece per row. K rho of the two rows stays in registers from
+// slice to slice and each row is the other's y neighbour: a slice of the pair
+// costs eight loads (two centres, two outer rows, four x neighbours), where a
+// thread per column needs ten. H = 1 (ZPAIR): padded coordinates are grid
+// coordinates + 1 and the halo repeats the nearest grid voxel; H = 0 (LINEAR,
+// and the max pass, which stores nothing): they are the grid's. A one-sided
+// difference is the central one with the missing neighbour replaced by the
+// voxel itself and the factor 1 instead of 1/2. Threads of the padding compute
+// a clamped voxel, which does not change a maximum and is not stored.
+template <int MODE, int H>  // 0: FP32 store, 1: FP16 max pass, 2: FP16 store
+__global__ void __launch_bounds__(256)
+    field_kernel(const float* __restrict__ rho, int nx, int ny, int nz, float K, unsigned width,
+                 int run, unsigned row, unsigned pair, void* __restrict__ out,
+                 unsigned* __restrict__ nz_bits, unsigned nz_words,
+                 unsigned* __restrict__ sparse,
+                 unsigned* __restrict__ max_bits, float* __restrict__ scales) {
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned jj = t / width, I = t - jj * width;
+    const int row_pairs = (ny + 2 * H + 1) / 2, slice_pairs = (nz + 2 * H + 1) / 2;
+    const bool valid = static_cast<int>(jj) < row_pairs && static_cast<int>(I) < nx + 2 * H;
+    const int i = min(max(static_cast<int>(I) - H, 0), nx - 1);
+    const int J0 = min(2 * static_cast<int>(jj), 2 * row_pairs - 2) - H, J1 = J0 + 1;
+    const int j0 = min(max(J0, 0), ny - 1), j1 = min(J1, ny - 1);
     float s_n = 1.0f, s_g = 1.0f;
     if (MODE == 2) {
         s_n = scale_of(max_bits[0]);
         s_g = scale_of(max_bits[1]);
     }
     const float rs_n = 1.0f / s_n, rs_g = 1.0f / s_g;  // exact: powers of two
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && MODE != 1) {
+    if (t == 0 && blockIdx.y == 0 && MODE != 1) {
         scales[0] = s_n;
         scales[1] = s_g;
+        if (H) *sparse = 0;  // free_mask_kernel, the next launch, may set it
+    }
+    const size_t sz = static_cast<size_t>(nx) * ny;
+    const float* r0 = rho + static_cast<size_t>(j0) * nx + i;
+    const float* r1 = rho + static_cast<size_t>(j1) * nx + i;
+    const float* ra = rho + static_cast<size_t>(max(j0 - 1, 0)) * nx + i;
+    const float* rd = rho + static_cast<size_t>(min(j1 + 1, ny - 1)) * nx + i;
+    const int xl = i > 0 ? -1 : 0, xh = i < nx - 1 ? 1 : 0;
+    const float fx = xl && xh ? 0.5f : 1.0f;
+    const float fy0 = j0 > 0 && j0 < ny - 1 ? 0.5f : 1.0f;
+    const float fy1 = j1 > 0 && j1 < ny - 1 ? 0.5f : 1.0f;
+    const bool first_row = J0 < 0, last_row = J1 >= ny;
+    const int kk0 = blockIdx.y * run, kk1 = min(kk0 + run, slice_pairs);
+    // dn = K rho, rounded by itself (an FMA with the difference that uses it would
+    // give a gradient that is not the stored dn's)
+    auto dn_of = [K](const float* p) { return __fmul_rn(K, __ldg(p)); };
+    auto at = [&](const float* p, int k) { return dn_of(p + static_cast<size_t>(k) * sz); };
+    // rows 0 and 1: p at slice s0 - 1, a at s0, b at s1, n at s1 + 1
+    float p0, p1, a0, a1;
+    {
+        const int k = max(2 * kk0 - H, 0);
+        p0 = at(r0, max(k - 1, 0));
+        p1 = at(r1, max(k - 1, 0));
+        a0 = at(r0, min(k, nz - 1));
+        a1 = at(r1, min(k, nz - 1));
     }
     float mn = 0.0f, mg = 0.0f;
-    // occupancy (the store passes): bit k - k0 set when this column stored a
-    // nonzero voxel at grid slice k (padded k + 1; the halo slices repeat
-    // slices 0 and nz - 1)
-    constexpr bool OCC = MODE != 1;
-    unsigned nzk = 0;
-    if (J < Hh) {
-        const int i = min(max(I - h, 0), nx - 1), j = min(max(J - h, 0), ny - 1);
-        const size_t sy = nx, sz = static_cast<size_t>(nx) * ny;
-        const float* col = rho + static_cast<size_t>(j) * sy + i;
-        const bool xl = i > 0, xh = i < nx - 1, yl = j > 0, yh = j < ny - 1;
-        float dprev = k0 > 0 ? K * __ldg(col + (k0 - 1) * sz) : 0.0f;
-        float dcur = K * __ldg(col + k0 * sz);
-#pragma unroll(MODE == 1 ? 4 : 2)
-        for (int k = k0; k < k1; ++k) {
-            const float* c = col + k * sz;
-            const float dnext = (k + 1 < nz) ? K * __ldg(c + sz) : 0.0f;
-            const float dxl = xl ? K * __ldg(c - 1) : 0.0f, dxh = xh ? K * __ldg(c + 1) : 0.0f;
-            const float dyl = yl ? K * __ldg(c - sy) : 0.0f, dyh = yh ? K * __ldg(c + sy) : 0.0f;
-            Cell e;
-            e.dn = dcur;
-            e.gx = !xl ? dxh - dcur : (!xh ? dcur - dxl : (dxh - dxl) * 0.5f);
-            e.gy = !yl ? dyh - dcur : (!yh ? dcur - dyl : (dyh - dyl) * 0.5f);
-            e.gz = (k == 0) ? dnext - dcur : (k == nz - 1 ? dcur - dprev : (dnext - dprev) * 0.5f);
-            const size_t o = h ? brick2_offset(I, J, k + 1, L.bx, L.bxy)
-                               : (static_cast<size_t>(k) * ny + j) * nx + i;
-            // z halo copies of the first and last slice
-            const bool zh = h && (k == 0 || k == nz - 1);
-            const size_t oh = zh ? brick2_offset(I, J, k == 0 ? 0 : nz + 1, L.bx, L.bxy) : 0;
-            bool nonzero = false;
-            if (MODE == 0) {
-                const float4 v = make_float4(e.dn, e.gx, e.gy, e.gz);
-                __stcs(static_cast<float4*>(out) + o, v);
-                if (zh) __stcs(static_cast<float4*>(out) + oh, v);
-                nonzero = v.x != 0.0f || v.y != 0.0f || v.z != 0.0f || v.w != 0.0f;
-            } else if (MODE == 1) {
-                mn = fmaxf(mn, fabsf(e.dn));
-                mg = fmaxf(mg, fmaxf(fabsf(e.gx), fmaxf(fabsf(e.gy), fabsf(e.gz))));
-            } else {
-                ushort4 q;  // the nearest half of value / s (exact products: s is a power of two)
-                q.x = __half_as_ushort(__float2half_rn(e.dn * rs_n));
-                q.y = __half_as_ushort(__float2half_rn(e.gx * rs_g));
-                q.z = __half_as_ushort(__float2half_rn(e.gy * rs_g));
-                q.w = __half_as_ushort(__float2half_rn(e.gz * rs_g));
-                const uint2 w = make_uint2(static_cast<unsigned>(q.x) | (static_cast<unsigned>(q.y) << 16),
-                                           static_cast<unsigned>(q.z) | (static_cast<unsigned>(q.w) << 16));
-                __stcs(static_cast<uint2*>(out) + o, w);
-                if (zh) __stcs(static_cast<uint2*>(out) + oh, w);
-                nonzero = ((w.x | w.y) & 0x7FFF7FFFu) != 0u;  // a half other than +-0
-            }
-            if (OCC) nzk |= static_cast<unsigned>(nonzero) << (k - k0);  // k - k0 < 16
-            dprev = dcur;
-            dcur = dnext;
+    for (int kk = kk0; kk < kk1; ++kk) {
+        const int K0 = 2 * kk - H, K1 = K0 + 1;  // grid slices of the pair
+        const int s0 = min(max(K0, 0), nz - 1), s1 = min(K1, nz - 1), sn = min(K1 + 1, nz - 1);
+        if (K0 >= nz) {  // the halo slice alone: again slice nz - 1, whose neighbour is nz - 2
+            p0 = at(r0, nz - 2);
+            p1 = at(r1, nz - 2);
         }
-    }
-    if (OCC && L.colbits && J < Hh) {
-        // one word per stored column and run (no atomics): bit t for grid
-        // slice k0 + t (padded k0 + t + 1), and in the last run bit nz - k0
-        // (at most 16) for the halo slice nz + 1, a copy of slice nz - 1; the
-        // halo slice 0, a copy of slice 0, is bit 0 of the first run
-        unsigned bits = nzk;
-        if (k1 == nz) bits |= ((nzk >> (nz - 1 - k0)) & 1u) << (nz - k0);
-        L.colbits[(static_cast<size_t>(blockIdx.y) * Hh + J) * L.pitch + I] = bits;
+        const float b0 = at(r0, s1), b1 = at(r1, s1);
+        const float n0 = at(r0, sn), n1 = at(r1, sn);
+        const float fz0 = s0 > 0 && s0 < nz - 1 ? 0.5f : 1.0f;
+        const float fz1 = s1 > 0 && s1 < nz - 1 ? 0.5f : 1.0f;
+        Voxel v00, v10, v01, v11;  // [row][slice]
+        v00.dn = a0;
+        v10.dn = a1;
+        v01.dn = b0;
+        v11.dn = b1;
+        // K0 < 0: the halo slice below slice 0, both of the pair are slice 0;
+        // K1 >= nz: both are slice nz - 1
+        v00.gz = ((K0 < 0 ? n0 : b0) - p0) * fz0;
+        v10.gz = ((K0 < 0 ? n1 : b1) - p1) * fz0;
+        v01.gz = (n0 - (K1 >= nz ? p0 : a0)) * fz1;
+        v11.gz = (n1 - (K1 >= nz ? p1 : a1)) * fz1;
+        {
+            const size_t z = static_cast<size_t>(s0) * sz;
+            const float oa = dn_of(ra + z), od = dn_of(rd + z);
+            v00.gx = (dn_of(r0 + z + xh) - dn_of(r0 + z + xl)) * fx;
+            v10.gx = (dn_of(r1 + z + xh) - dn_of(r1 + z + xl)) * fx;
+            v00.gy = ((first_row ? od : a1) - oa) * fy0;
+            v10.gy = (od - (last_row ? oa : a0)) * fy1;
+        }
+        {
+            const size_t z = static_cast<size_t>(s1) * sz;
+            const float oa = dn_of(ra + z), od = dn_of(rd + z);
+            v01.gx = (dn_of(r0 + z + xh) - dn_of(r0 + z + xl)) * fx;
+            v11.gx = (dn_of(r1 + z + xh) - dn_of(r1 + z + xl)) * fx;
+            v01.gy = ((first_row ? od : b1) - oa) * fy0;
+            v11.gy = (od - (last_row ? oa : b0)) * fy1;
+        }
+        if (MODE == 1) {
+            auto peak = [&](const Voxel& v) {
+                mn = fmaxf(mn, fabsf(v.dn));
+                mg = fmaxf(mg, fmaxf(fabsf(v.gx), fmaxf(fabsf(v.gy), fabsf(v.gz))));
+            };
+            peak(v00);
+            peak(v10);
+            peak(v01);
+            peak(v11);
+        } else if (H == 0) {
+            if (valid) {
+                const size_t o = (static_cast<size_t>(K0) * ny + J0) * nx + I;
+                uint4* to = static_cast<uint4*>(out) + o;
+                __stcs(to, pack32(v00));
+                if (J1 < ny) __stcs(to + nx, pack32(v10));
+                if (K1 < nz) __stcs(to + sz, pack32(v01));
+                if (J1 < ny && K1 < nz) __stcs(to + sz + nx, pack32(v11));
+            }
+        } else {
+            const unsigned J = 2 * jj, slice = 2 * static_cast<unsigned>(kk);
+            const bool valid1 = valid && static_cast<int>(J) + 1 < ny + 2;
+            const size_t o = static_cast<size_t>(kk) * pair + J * row + 2 * I;
+            bool z00, z10, z01, z11;  // holds only +-0
+            if (MODE == 0) {
+                const uint4 w00 = pack32(v00), w01 = pack32(v01);
+                const uint4 w10 = pack32(v10), w11 = pack32(v11);
+                auto zero = [](uint4 w) { return ((w.x | w.y | w.z | w.w) & 0x7FFFFFFFu) == 0u; };
+                z00 = zero(w00);
+                z01 = zero(w01);
+                z10 = zero(w10);
+                z11 = zero(w11);
+                uint4* to = static_cast<uint4*>(out) + o;
+                if (valid) store32(to, w00, w01);
+                if (valid1) store32(to + row, w10, w11);
+            } else {
+                const uint2 w00 = pack16(v00, rs_n, rs_g), w01 = pack16(v01, rs_n, rs_g);
+                const uint2 w10 = pack16(v10, rs_n, rs_g), w11 = pack16(v11, rs_n, rs_g);
+                auto zero = [](uint2 w) { return ((w.x | w.y) & 0x7FFF7FFFu) == 0u; };
+                z00 = zero(w00);
+                z01 = zero(w01);
+                z10 = zero(w10);
+                z11 = zero(w11);
+                uint2* to = static_cast<uint2*>(out) + o;
+                if (valid) __stcs(reinterpret_cast<uint4*>(to), make_uint4(w00.x, w00.y, w01.x, w01.y));
+                if (valid1)
+                    __stcs(reinterpret_cast<uint4*>(to + row), make_uint4(w10.x, w10.y, w11.x, w11.y));
+            }
+            // nonzero bits, a word per row and slice (width is a multiple of
+            // 32: a warp is one word of one pair of rows); the padding counts
+            // as nonzero
+            const unsigned n00 = __ballot_sync(0xffffffffu, !(valid && z00));
+            const unsigned n10 = __ballot_sync(0xffffffffu, !(valid1 && z10));
+            const unsigned n01 = __ballot_sync(0xffffffffu, !(valid && z01));
+            const unsigned n11 = __ballot_sync(0xffffffffu, !(valid1 && z11));
+            const unsigned lane = threadIdx.x & 31;
+            if (lane < 4 && static_cast<int>(jj) < row_pairs) {
+                const unsigned word = lane & 2 ? (lane & 1 ? n11 : n01) : (lane & 1 ? n10 : n00);
+                const unsigned rows = 2 * static_cast<unsigned>(row_pairs);
+                nz_bits[(static_cast<size_t>(slice + (lane >> 1)) * rows + J + (lane & 1)) * nz_words +
+                        (I >> 5)] = word;
+            }
+        }
+        p0 = b0;
+        p1 = b1;
+        a0 = n0;
+        a1 = n1;
     }
     if (MODE == 1) {  // block maximum, then one atomic per block
-        for (int o = 16; o > 0; o >>= 1) {
-            mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-            mg = fmaxf(mg, __shfl_xor_sync(0xffffffffu, mg, o));
+        for (int d = 16; d > 0; d >>= 1) {
+            mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, d));
+            mg = fmaxf(mg, __shfl_xor_sync(0xffffffffu, mg, d));
         }
         __shared__ float sn[8], sg[8];
         if ((threadIdx.x & 31) == 0) {
@@ -184,84 +249,78 @@ __global__ void __launch_bounds__(256, 8) field_column_kernel(const float* __res
     }
 }
 
-// The free-corner mask from the store pass's column words: one bit per
-// stored element of the BRICK2 layout (bit b & 7 of byte b >> 3 for element
-// b, i.e. a byte per brick, bit = slot), set when the voxel at padded (I, J,
-// K) and its +1 neighbours on each axis (the eight corners of the trilinear
-// cell whose first corner it is) hold no stored nonzero value. A thread takes
-// the bricks (bx, by, bz) of one brick column (bx, by) whose slices lie in
-// run r: bz = 8r + 1 .. 8r + 8 (padded slices 16r + 2 .. 16r + 17), and bz =
-// 0 too when r = 0. It reads the column words of the 3 x 3 stored columns
-// I = 2bx .. 2bx + 2, J = 2by .. 2by + 2 for runs r and r + 1 (zero beyond the
-// stored columns and runs), shifted so that bit j stands for padded slice
-// 16r + j (bit 0 only needed for r = 0: the halo slice 0), ORs neighbouring
-// columns and rows for the four (x, y) slot parities and neighbouring slices
-// for z, and stores each brick's byte (one writer per byte, no atomics).
-__global__ void free_mask_kernel(const uint32_t* __restrict__ colbits, int pitch, int H, int runs,
-                                 unsigned nbx, unsigned nby, unsigned nbz,
-                                 uint8_t* __restrict__ fr) {
-    const unsigned bx = blockIdx.x * 32 + threadIdx.x;
-    const unsigned by = blockIdx.y * blockDim.y + threadIdx.y;
-    const int r = static_cast<int>(blockIdx.z);
-    if (bx >= nbx || by >= nby) return;
-    unsigned xo[3][2];  // per row: columns (2bx, 2bx+1) and (2bx+1, 2bx+2) ORed
+// A warp's stretch of the mask (1024 elements) with at least this many free
+// ones makes the volume sparse: the march then tests the mask at each sample.
+// Below it, over the whole volume, the test costs a load's latency and six
+// instructions a sample and saves next to nothing (720p view of a 192x160x224
+// turbulence volume without empty space: 194 us with it, 182 without).
+constexpr unsigned kSparseFree = 128;
+
+// The free-corner mask from the store pass's nonzero bits, a word (32
+// consecutive elements: 16 columns of a row of a pair of slices, or the end of
+// one row and the start of the next) per thread. Column I of row J, slice K is
+// free when none of columns I, I + 1 of rows J, J + 1 of slices K, K + 1 holds a
+// nonzero value; whatever lies beyond the stored rows and columns counts as
+// nonzero.
+__global__ void __launch_bounds__(256)
+    free_mask_kernel(const unsigned* __restrict__ nz, unsigned nz_words, unsigned rows,
+                     unsigned pairs, unsigned row, unsigned pair, unsigned words,
+                     unsigned* __restrict__ fr, unsigned* __restrict__ sparse) {
+    const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned free_bits = 0;
+    if (g < words) {
+        // 32 columns from column c of a row's nonzero bits
+        auto columns = [&](unsigned slice, unsigned J, unsigned c) {
+            if (slice >= 2 * pairs || J >= rows) return 0xFFFFFFFFu;
+            const unsigned* w = nz + (static_cast<size_t>(slice) * rows + J) * nz_words;
+            const unsigned i = c >> 5;
+            const unsigned lo = i < nz_words ? __ldg(w + i) : 0xFFFFFFFFu;
+            const unsigned hi = i + 1 < nz_words ? __ldg(w + i + 1) : 0xFFFFFFFFu;
+            return __funnelshift_r(lo, hi, c);
+        };
+        auto spread = [](unsigned x) {  // bit i of the low half to bit 2 i
+            x = (x | (x << 8)) & 0x00FF00FFu;
+            x = (x | (x << 4)) & 0x0F0F0F0Fu;
+            x = (x | (x << 2)) & 0x33333333u;
+            return (x | (x << 1)) & 0x55555555u;
+        };
+        unsigned kk = 32u * g / pair, at = 32u * g - kk * pair;  // elements: below 2^32
+        for (unsigned done = 0; done < 32u && kk < pairs;) {
+            const unsigned J = at / row, e = at - J * row;  // e is even
+            const unsigned n = min(32u - done, min(row - e, pair - at));
+            unsigned busy[3];
 #pragma unroll
-    for (int jr = 0; jr < 3; ++jr) {
-        const int J = 2 * static_cast<int>(by) + jr;
-        unsigned c[3] = {0u, 0u, 0u};
-        if (J < H) {
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (r + q >= runs) break;
-                const uint32_t* row = colbits + (static_cast<size_t>(r + q) * H + J) * pitch;
-#pragma unroll
-                for (int ic = 0; ic < 3; ++ic) {
-                    const unsigned I = 2 * bx + static_cast<unsigned>(ic);
-                    if (I < static_cast<unsigned>(pitch)) {
-                        const unsigned w = __ldg(row + I);
-                        // run r: bit t -> padded 16r + 1 + t; run r + 1: 16r + 17 + t
-                        c[ic] |= q == 0 ? (w << 1) | (r == 0 ? (w & 1u) : 0u) : (w << 17);
-                    }
-                }
+            for (unsigned z = 0; z < 3; ++z) {
+                const unsigned a = columns(2 * kk + z, J, e >> 1) | columns(2 * kk + z, J + 1, e >> 1);
+                busy[z] = a | (a >> 1);
+            }
+            const unsigned b = spread((busy[0] | busy[1]) & 0xFFFFu) |
+                               (spread((busy[1] | busy[2]) & 0xFFFFu) << 1);
+            free_bits |= (~b & (0xFFFFFFFFu >> (32u - n))) << done;
+            done += n;
+            at += n;
+            if (at == pair) {
+                at = 0;
+                ++kk;
             }
         }
-        xo[jr][0] = c[0] | c[1];
-        xo[jr][1] = c[1] | c[2];
+        fr[g] = free_bits;
     }
-    unsigned busy[2][2];  // [y parity][x parity]: bit j, slice 16r + j or 16r + j + 1 occupied
-#pragma unroll
-    for (int sy = 0; sy < 2; ++sy)
-#pragma unroll
-        for (int sx = 0; sx < 2; ++sx) {
-            const unsigned o = xo[sy][sx] | xo[sy + 1][sx];
-            busy[sy][sx] = o | (o >> 1);
-        }
-    const size_t nbxy = static_cast<size_t>(nbx) * nby;
-    const size_t col = static_cast<size_t>(by) * nbx + bx;
-    for (int m = (r == 0) ? 0 : 1; m <= 8; ++m) {
-        const unsigned bz = 8u * static_cast<unsigned>(r) + static_cast<unsigned>(m);
-        if (bz >= nbz) break;
-        unsigned byte = 0;
-#pragma unroll
-        for (int sz = 0; sz < 2; ++sz)
-#pragma unroll
-            for (int sy = 0; sy < 2; ++sy)
-#pragma unroll
-                for (int sx = 0; sx < 2; ++sx)
-                    byte |= ((~busy[sy][sx] >> (2 * m + sz)) & 1u) << (sx | (sy << 1) | (sz << 2));
-        fr[bz * nbxy + col] = static_cast<uint8_t>(byte);
-    }
+    const unsigned free_here = __reduce_add_sync(0xffffffffu, __popc(free_bits));
+    if (free_here >= kSparseFree && (threadIdx.x & 31) == 0) *sparse = 1;
 }
 
-__global__ void export_kernel(const void* __restrict__ data, int storage, OutLayout L, int nx,
-                              int ny, int nz, const float* __restrict__ scales,
+__global__ void export_kernel(const void* __restrict__ data, int storage, unsigned row,
+                              unsigned pair, int nx, int ny, const float* __restrict__ scales,
                               float4* __restrict__ dst) {
     const int i = blockIdx.x * 32 + threadIdx.x;
     const int j = blockIdx.y * 8 + threadIdx.y;
     const int k = blockIdx.z;
     if (i >= nx || j >= ny) return;
     const size_t v = (static_cast<size_t>(k) * ny + j) * nx + i;
-    const size_t src = out_index(L, i, j, k, nx, ny);
+    const unsigned Kp = k + 1;
+    const size_t src = static_cast<size_t>(Kp >> 1) * pair + static_cast<size_t>(j + 1) * row +
+                       2u * (i + 1) + (Kp & 1u);
     if (storage == HH_STORE_FP32) {
         dst[v] = reinterpret_cast<const float4*>(data)[src];
     } else {
@@ -278,50 +337,58 @@ __global__ void export_kernel(const void* __restrict__ data, int storage, OutLay
 
 cudaError_t launch_field(const float* rho, int nx, int ny, int nz, float K, hh_volume_s* vol,
                          cudaStream_t s) {
-    // 256 threads per block over the stored (x, y) columns; blockIdx.y picks
-    // the z run. The FP16 max pass covers the grid columns only (no halo).
-    const int h2 = vol->layout == HH_LAYOUT_BRICK2 ? 2 : 0;
+    // 256 threads per block over (row pair, column), rows padded to whole
+    // warps; blockIdx.y picks the run of slice pairs: eight, or fewer where
+    // that leaves the chip with less than four blocks an SM
+    const bool halo = vol->layout == HH_LAYOUT_ZPAIR;
     const dim3 block(256);
-    const dim3 grid(static_cast<unsigned>((static_cast<int64_t>(nx + h2) * (ny + h2) + 255) / 256),
-                    (nz + FIELD_ZRUN - 1) / FIELD_ZRUN);
-    const dim3 grid_max(static_cast<unsigned>((static_cast<int64_t>(nx) * ny + 255) / 256),
-                        (nz + FIELD_ZRUN - 1) / FIELD_ZRUN);
-    const bool masks = vol->layout == HH_LAYOUT_BRICK2 && vol->colbits_dev != nullptr;
-    const int pitch = (nx + 2 + 3) & ~3;
-    const int runs = (nz + FIELD_ZRUN - 1) / FIELD_ZRUN;
-    const OutLayout L{vol->layout, vol->bx, vol->bxy, masks ? vol->colbits_dev : nullptr, pitch};
+    auto grid_of = [&](int h, int& run) {
+        const unsigned row_pairs = (ny + 2 * h + 1) / 2, pairs = (nz + 2 * h + 1) / 2;
+        const unsigned width = (nx + 2 * h + 31) / 32 * 32;
+        const unsigned blocks = (row_pairs * width + 255) / 256;
+        run = 8;
+        while (run > 1 && blocks * ((pairs + run - 1) / run) < 608) run /= 2;
+        return dim3(blocks, (pairs + run - 1) / run);
+    };
+    int run = 0;
+    const unsigned width = (nx + (halo ? 2 : 0) + 31) / 32 * 32;
+    const dim3 grid = grid_of(halo ? 1 : 0, run);
     cudaError_t e = cudaSuccess;
     if (vol->storage == HH_STORE_FP32) {
-        field_column_kernel<0><<<grid, block, 0, s>>>(rho, nx, ny, nz, K, L, vol->data, nullptr,
-                                                      vol->scales_dev);
+        (halo ? field_kernel<0, 1> : field_kernel<0, 0>)<<<grid, block, 0, s>>>(
+            rho, nx, ny, nz, K, width, run, vol->row, vol->pair, vol->data, vol->nz_dev,
+            vol->nz_words, vol->sparse_dev, nullptr, vol->scales_dev);
         count_launch();
     } else {
         e = cudaMemsetAsync(vol->max_dev, 0, 2 * sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
-        field_column_kernel<1><<<grid_max, block, 0, s>>>(rho, nx, ny, nz, K, L, nullptr,
-                                                          vol->max_dev, vol->scales_dev);
-        field_column_kernel<2><<<grid, block, 0, s>>>(rho, nx, ny, nz, K, L, vol->data,
+        int max_run = 0;
+        const dim3 max_grid = grid_of(0, max_run);
+        field_kernel<1, 0><<<max_grid, block, 0, s>>>(rho, nx, ny, nz, K, (nx + 31) / 32 * 32,
+                                                      max_run, 0, 0, nullptr, nullptr, 0, nullptr,
                                                       vol->max_dev, vol->scales_dev);
+        field_kernel<2, 1><<<grid, block, 0, s>>>(rho, nx, ny, nz, K, width, run, vol->row,
+                                                  vol->pair, vol->data, vol->nz_dev, vol->nz_words,
+                                                  vol->sparse_dev, vol->max_dev, vol->scales_dev);
         count_launch(2);
     }
-    if (masks) {
-        const unsigned nby = vol->bxy / vol->bx;
-        const dim3 mblock(32, 8);
-        const dim3 mgrid((vol->bx + 31) / 32, (nby + 7) / 8, static_cast<unsigned>(runs));
-        free_mask_kernel<<<mgrid, mblock, 0, s>>>(vol->colbits_dev, pitch, ny + 2, runs, vol->bx,
-                                                  nby, vol->bz,
-                                                  reinterpret_cast<uint8_t*>(vol->free_dev));
+    if (halo) {
+        const unsigned rows = (ny + 3) / 2 * 2, pairs = (nz + 3) / 2;
+        const unsigned words = static_cast<unsigned>((static_cast<size_t>(vol->pair) * pairs + 31) / 32);
+        free_mask_kernel<<<(words + 255) / 256, block, 0, s>>>(vol->nz_dev, vol->nz_words, rows,
+                                                               pairs, vol->row, vol->pair, words,
+                                                               vol->free_dev, vol->sparse_dev);
         count_launch();
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_export(const hh_volume_s* vol, float4* dst, cudaStream_t s) {
+    if (vol->layout != HH_LAYOUT_ZPAIR) return cudaErrorInvalidValue;
     const dim3 block(32, 8);
     const dim3 grid((vol->nx + 31) / 32, (vol->ny + 7) / 8, vol->nz);
-    const OutLayout L{vol->layout, vol->bx, vol->bxy, nullptr, 0};
-    export_kernel<<<grid, block, 0, s>>>(vol->data, vol->storage, L, vol->nx, vol->ny, vol->nz,
-                                         vol->scales_dev, dst);
+    export_kernel<<<grid, block, 0, s>>>(vol->data, vol->storage, vol->row, vol->pair, vol->nx,
+                                         vol->ny, vol->scales_dev, dst);
     count_launch();
     return cudaGetLastError();
 }

@@ -15,51 +15,57 @@
 #define HH_FP16_CODE_MAX 16384.0f
 
 // Volume layouts.
-//  LINEAR: x fastest, index (k*ny + j)*nx + i (the export / interchange layout).
-//  BRICK2: 2x2x2 micro-bricks over the grid with a one-voxel halo: voxel
-//          (i,j,k) sits at padded coordinates (I,J,K) = (i+1, j+1, k+1), and
-//          the halo (I = 0 or n+1 on some axis) holds a copy of the nearest
-//          grid voxel, so a trilinear sample clamped to the edge needs no
-//          index clamps. Brick (I>>1, J>>1, K>>1) in x-fastest order over
-//          ceil((n+2)/2) bricks per axis; inside a brick the voxel sits at
-//          slot (I&1) | (J&1)<<1 | (K&1)<<2. One FP32 brick is one 128-byte
-//          line, and the eight corners of any trilinear cell occupy eight
-//          different slots, i.e. eight different 16-byte L1 bank groups, so a
-//          warp's corner loads spread over all banks whatever the view
-//          direction (the linear layout puts every y/z neighbour of a
-//          power-of-two grid into the same bank group).
-enum { HH_LAYOUT_LINEAR = 0, HH_LAYOUT_BRICK2 = 1 };
+//  LINEAR: x fastest, element (k*ny + j)*nx + i (the export / interchange
+//          layout).
+//  ZPAIR: the grid with a one-voxel halo: voxel (i,j,k) sits at padded
+//          coordinates (I,J,K) = (i+1, j+1, k+1), and the halo (0 or n+1 on
+//          some axis) holds a copy of the nearest grid voxel, so a trilinear
+//          sample clamped to the edge needs no index clamps. Two slices are
+//          interleaved: element (K>>1)*pair + J*row + 2*I + (K&1). A cell then
+//          needs one base element and one select (the step to the next slice);
+//          the next row and the next column are constant strides. Against 2x2x2
+//          bricks (a select per axis, an address per corner) the march of a
+//          256^3 FP32 1080p frame at h_max takes 330 instead of 359 us, of a
+//          384^3 FP16 4K view 1657 instead of 1883; a plain x-fastest order
+//          takes 333 and 1604, but its lines of eight voxels in a row spread a
+//          cell over more of them (32 views of a 512^3 FP16 volume: 11.1 ms
+//          against 10.0, and 10.1 for the bricks).
+//          row = 12 and pair = 2 (mod 16): the eight corners of any cell lie
+//          in eight different 16-byte L1 bank groups (8-byte ones on FP16
+//          storage), and so do the cells around it as far as that goes; of ten
+//          residue pairs this one was the fastest on the 512^3 views (10.0
+//          against 10.1-10.8 ms) and no slower on the others.
+enum { HH_LAYOUT_LINEAR = 0, HH_LAYOUT_ZPAIR = 1 };
 
-// Bricks along an axis of n voxels in the BRICK2 layout (halo included).
-__host__ __device__ __forceinline__ unsigned brick2_count(int n) {
-    return static_cast<unsigned>((n + 3) / 2);
+// ZPAIR strides in elements: of a row, and of a pair of slices. (A grid within
+// the size limit of the entry points has less than 2^32 elements.)
+inline unsigned zpair_row(int nx) { return (2u * static_cast<unsigned>(nx) + 7u) / 16u * 16u + 12u; }
+inline unsigned zpair_pair(int nx, int ny) {
+    return (zpair_row(nx) * (static_cast<unsigned>(ny) + 2u) + 13u) / 16u * 16u + 2u;
 }
-
-// Element of padded coordinates (I, J, K) in the BRICK2 layout.
-__host__ __device__ __forceinline__ unsigned brick2_offset(unsigned i, unsigned j, unsigned k,
-                                                           unsigned bx, unsigned bxy) {
-    return (((k >> 1) * bxy + (j >> 1) * bx + (i >> 1)) << 3) | ((k & 1u) << 2) |
-           ((j & 1u) << 1) | (i & 1u);
-}
-
 
 struct hh_volume_s {
     int nx, ny, nz;
     int storage;        // hh_storage
     int layout;         // HH_LAYOUT_*
-    unsigned bx, bxy;   // BRICK2: bricks along x, bricks per xy plane
+    unsigned row, pair; // ZPAIR strides (elements)
     float h_kernel;
     void* data;         // float4 (FP32) or ushort4 of halves (FP16) per voxel
-    size_t bytes;       // bytes of data (BRICK2: halo of one voxel, axes padded to even)
-    // BRICK2 free-corner mask, one bit per stored element in the layout's own
-    // order (bit b & 31 of word b >> 5 for element b), at data + bytes in the
-    // same allocation: set when the element's voxel and its +1 neighbours on
-    // each axis hold no stored nonzero value, so that a sample whose first
-    // corner is that voxel reads eight zeros. Null for LINEAR volumes.
-    unsigned bz;           // bricks along z
-    size_t mask_words;     // 32-bit words of the mask
+    size_t bytes;       // the packed field's bytes as reported: grid and halo, axes padded to even
+    // ZPAIR: the free-corner mask and its build scratch follow the data in the
+    // same allocation. free_dev: one bit per element in the layout's own order
+    // (bit b & 31 of word b >> 5 for element b), set when the element's voxel
+    // and its +1 neighbours on each axis hold no stored nonzero value, so that
+    // a sample whose first corner is that voxel reads eight zeros. nz_dev: one
+    // bit per voxel, rows of nz_words words (bit I & 31 of word (K * (ny + 2) +
+    // J) * nz_words + (I >> 5)), set when the voxel holds a nonzero value. sparse_dev: nonzero when some
+    // stretch of the mask is worth testing (see free_mask_kernel). Null for
+    // LINEAR volumes.
+    size_t mask_off;    // bytes from data to free_dev
+    unsigned nz_words;
     unsigned* free_dev;
-    uint32_t* colbits_dev; // scratch of the mask build: a word per stored column and z run
+    unsigned* nz_dev;
+    unsigned* sparse_dev;
     float* scales_dev;  // [2] = {s_n, s_g} on the device (1, 1 for FP32)
     unsigned* max_dev;  // [2] = bit patterns of max|dn|, max|g| (FP16 build)
     float* rho_dev;     // density scratch for particle builds (nullable)
@@ -127,8 +133,9 @@ int build_view_table(const hh_camera* cams, const hh_view_out* outs, int n, int 
 // host-mapped memory. Jobs are numbered from 0 since the queue's last reset;
 // the host resets the queue only while no worker runs.
 struct ServeJob {
-    const void* vol;      // the frame's volume data (BRICK2)
+    const void* vol;      // the frame's volume data (ZPAIR)
     const float* scales;  // its FP16 scales on the device
+    const unsigned* sparse;  // whether its free-corner mask is worth testing
     int view_begin;       // first record of the job in the view table
     int n_views;
     int n_tiles;          // tiles of all its views (view tile_begin is job-relative)

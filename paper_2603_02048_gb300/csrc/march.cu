@@ -24,13 +24,14 @@
 //
 // Layout: a block of 128 threads covers a 16x8 pixel tile; each warp an 8x4
 // sub-tile, so the rays of a warp stay close in the volume and their eight
-// corner fetches per step share cache lines in L1. The volume is stored in
-// 2x2x2 micro-bricks (BRICK2) with a one-voxel halo of edge copies: the
-// bricks spread the distinct voxels of a warp's corner load over all L1 bank
-// groups, and the halo lets a sample in the box skip every index clamp.
+// corner fetches per step share cache lines in L1. The volume is stored with
+// its slices interleaved in pairs (ZPAIR) and a one-voxel halo of edge copies:
+// the order spreads the distinct voxels of a warp's corner load over the L1
+// bank groups at a cost of few address instructions, and the halo lets a
+// sample in the box skip every index clamp.
 // A sample whose eight corners are all zero (its first corner marked in the
 // volume's free-corner mask, built with the volume) is read as zero from one
-// bit of that mask instead of eight brick loads, and the Eq. 16 step then
+// bit of that mask instead of eight voxel loads, and the Eq. 16 step then
 // takes n = 1, g_perp = 0 and their step length without the arithmetic (a
 // warp whose lanes all sample zero skips it); every step is still taken with
 // the values the general branch would compute, so the results do not depend
@@ -41,6 +42,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "hh_internal.h"
@@ -63,9 +65,10 @@ constexpr float kPi = 3.14159265358979323846f;
 struct VolArgs {
     const void* vol;
     const float* scales;
+    const unsigned* sparse;  // whether the volume's free-corner mask is worth testing
     int nx, ny, nz;
-    unsigned bx, bxy;   // BRICK2 bricks along x and per xy plane
-    unsigned by8, bz8;  // BRICK2 strides (in elements) of one brick step in y and z
+    unsigned row, half_pair;      // ZPAIR strides of a row, and half of a pair of slices (elements)
+    unsigned row_bytes, up_bytes; // a row, and the step from an odd slice to the next - 1 element
     unsigned long long mask_off;  // bytes from a volume's data to its free-corner mask
     float bias;         // power of two above every coordinate and step
     float bias_u;       // bias - 1/2: (hi - bias_u) + lo is the lattice coordinate
@@ -154,6 +157,7 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return r;
 }
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 // a + t (b - a) on both halves of a float4 (t duplicated in tt).
 __device__ __forceinline__ float4 lerp4x2(float4 a, float4 b, float2 tt) {
     const float2 lo = fma2(tt, sub2(make_float2(b.x, b.y), make_float2(a.x, a.y)),
@@ -171,7 +175,7 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 }
 
 // Lattice cell and weight along one axis from the lattice coordinate u =
-// position + 1/2, the halo coordinate of the BRICK2 layout (the centre of
+// position + 1/2, the halo coordinate of the ZPAIR layout (the centre of
 // grid voxel i at u = i + 1; the march carries u, not the position):
 // i0 = floor(u), f = u - i0. A position in [0, n] has u in [0.5, n + 0.5], so
 // both corners i0, i0 + 1 lie in the padded axis [0, n + 1], and the halo
@@ -187,9 +191,6 @@ __device__ __forceinline__ void axis_cell(float u, int n, int& i0, float& f) {
     f = u - fl;
 }
 
-__device__ __forceinline__ float4 ld_fp32(const float4* __restrict__ v, unsigned i) {
-    return __ldg(v + i);
-}
 // x-lerp of two FP16 corners read raw (four halves each), in FP32: the first
 // corner converted, the second converted inside the subtraction
 // (sub.rn.f32.f16: one rounding, as converting first and subtracting in FP32),
@@ -221,9 +222,18 @@ __device__ __forceinline__ float4 xlerp_fp16(uint2 a, uint2 b, float2 tt) {
 __device__ unsigned long long g_bounds_violations;
 #endif
 
+// How a kernel addresses the volume. ADDR_BASE: at V.vol, below 4 GiB, as
+// 32-bit byte offsets from base addresses the whole grid shares, which cost a
+// load no address arithmetic (FP16 384^3 4K view: 1733 against 1657 us).
+// ADDR_ANY: at a pointer of the caller's (the serving worker's jobs) or of any
+// size, with 64-bit addresses.
+enum { ADDR_BASE = 0, ADDR_ANY = 1 };
+
 // Returns false, leaving s unset, for a sample whose eight corners are all
-// zero (the zero sample).
-template <int STORAGE, bool CLAMP>
+// zero (the zero sample), read off the free-corner mask. MASK = false (volumes
+// not worth testing) never asks: the general arithmetic on eight zeros gives
+// the zero sample's values.
+template <int STORAGE, int ADDR, bool MASK, bool CLAMP>
 __device__ __forceinline__ bool fetch_nonzero(const VolArgs& A, const void* __restrict__ vol,
                                               float3 u, uint32_t& flags, Sample& s) {
     int ix, iy, iz;
@@ -245,73 +255,73 @@ __device__ __forceinline__ bool fetch_nonzero(const VolArgs& A, const void* __re
 #else
     (void)flags;
 #endif
-    // BRICK2 element of corner (ix, iy, iz): brick b >> 3, slot b & 7.
-    const unsigned b = brick2_offset(ix, iy, iz, A.bx, A.bxy);
-    // A sample whose eight corners are all zero is the zero sample: read from
-    // the volume's free-corner mask (bit b & 31 of word b >> 5; the funnel
-    // shift takes the shift count mod 32) instead of the bricks.
-    {
-        const unsigned* fm =
-            reinterpret_cast<const unsigned*>(static_cast<const char*>(vol) + A.mask_off);
-        const unsigned w = __ldg(fm + (b >> 5));
+    // ZPAIR element of corner (ix, iy, iz): (iz >> 1) pair + iy row + 2 ix + (iz
+    // & 1), the pair's half taken out by the parity
+    const unsigned odd = static_cast<unsigned>(iz) & 1u;
+    const unsigned b = static_cast<unsigned>(iz) * A.half_pair +
+                       static_cast<unsigned>(iy) * A.row + 2u * static_cast<unsigned>(ix) -
+                       odd * (A.half_pair - 1u);
+    // the zero sample's bit: b & 31 of word b >> 5 (the funnel shift takes the
+    // shift count mod 32)
+    const char* base = static_cast<const char*>(ADDR == ADDR_BASE ? A.vol : vol);
+    if (MASK) {
+        const unsigned w = __ldg(reinterpret_cast<const unsigned*>(base + A.mask_off) + (b >> 5));
         if (__funnelshift_r(w, w, b) & 1u) return false;
     }
-    // The steps to the other corners: +1 in x stays in the brick (slot +1)
-    // when ix is even, else it moves to the next brick (slot -1, brick +1:
-    // +7); likewise y (+2 or by8 - 2) and z (+4 or bz8 - 4).
-    const unsigned dx = (ix & 1) ? 7u : 1u;
-    const unsigned dy = (iy & 1) ? A.by8 - 2u : 2u;
-    const unsigned dz = (iz & 1) ? A.bz8 - 4u : 4u;
-    const unsigned b010 = b + dy, b001 = b + dz, b011 = b001 + dy;
-    float4 v000, v100, v010, v110, v001, v101, v011, v111;
-    if (STORAGE == HH_STORE_FP32) {
-        const float4* V = static_cast<const float4*>(vol);
-        v000 = ld_fp32(V, b);
-        v100 = ld_fp32(V, b + dx);
-        v010 = ld_fp32(V, b010);
-        v110 = ld_fp32(V, b010 + dx);
-        v001 = ld_fp32(V, b001);
-        v101 = ld_fp32(V, b001 + dx);
-        v011 = ld_fp32(V, b011);
-        v111 = ld_fp32(V, b011 + dx);
+    // The other corners: the next column is 2 elements on, the next row `row`,
+    // the next slice 1 for an even slice, else pair - 1.
+    using V = typename std::conditional<STORAGE == HH_STORE_FP32, float4, uint2>::type;
+    constexpr unsigned size = sizeof(V);
+    const unsigned up = odd * A.up_bytes + size;
+    const V *c00, *c10, *c01, *c11;  // corners (ix, iy + 0 or 1, iz + 0 or 1)
+    if (ADDR == ADDR_BASE) {
+        const char* next = base + A.row_bytes;
+        const unsigned at = b * size, above = at + up;
+        c00 = reinterpret_cast<const V*>(base + at);
+        c10 = reinterpret_cast<const V*>(next + at);
+        c01 = reinterpret_cast<const V*>(base + above);
+        c11 = reinterpret_cast<const V*>(next + above);
+    } else {
+        c00 = reinterpret_cast<const V*>(base) + b;
+        c01 = reinterpret_cast<const V*>(reinterpret_cast<const char*>(c00) + up);
+        c10 = reinterpret_cast<const V*>(reinterpret_cast<const char*>(c00) + A.row_bytes);
+        c11 = reinterpret_cast<const V*>(reinterpret_cast<const char*>(c01) + A.row_bytes);
     }
     float4 c;
-    if (STORAGE == HH_STORE_FP16_SCALED) {
-    // FP16 storage: lerps along x (the second corner converted inside the
-    // subtraction), then y, then z with packed FP32x2 arithmetic, two channels
-    // per instruction (measured 8 % faster there; on FP32 storage the 8-weight
-    // form below is faster)
-    const uint2* V = static_cast<const uint2*>(vol);
-    const uint2 r000 = __ldg(V + b), r100 = __ldg(V + b + dx);
-    const uint2 r010 = __ldg(V + b010), r110 = __ldg(V + b010 + dx);
-    const uint2 r001 = __ldg(V + b001), r101 = __ldg(V + b001 + dx);
-    const uint2 r011 = __ldg(V + b011), r111 = __ldg(V + b011 + dx);
-    const float2 tx = make_float2(fx, fx), ty = make_float2(fy, fy), tz = make_float2(fz, fz);
-    c = lerp4x2(lerp4x2(xlerp_fp16(r000, r100, tx), xlerp_fp16(r010, r110, tx), ty),
-                lerp4x2(xlerp_fp16(r001, r101, tx), xlerp_fp16(r011, r111, tx), ty), tz);
+    if constexpr (STORAGE == HH_STORE_FP16_SCALED) {
+        // lerps along x (the second corner converted inside the subtraction),
+        // then y, then z with packed FP32x2 arithmetic, two channels per
+        // instruction (measured 8 % faster there; on FP32 storage the 8-weight
+        // form below is faster)
+        const uint2 r000 = __ldg(c00), r100 = __ldg(c00 + 2), r010 = __ldg(c10), r110 = __ldg(c10 + 2);
+        const uint2 r001 = __ldg(c01), r101 = __ldg(c01 + 2), r011 = __ldg(c11), r111 = __ldg(c11 + 2);
+        const float2 tx = dup(fx), ty = dup(fy), tz = dup(fz);
+        c = lerp4x2(lerp4x2(xlerp_fp16(r000, r100, tx), xlerp_fp16(r010, r110, tx), ty),
+                    lerp4x2(xlerp_fp16(r001, r101, tx), xlerp_fp16(r011, r111, tx), ty), tz);
     } else {
-    // the standard 8-corner weights
-    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-    const float w00 = gy * gz, w10 = fy * gz, w01 = gy * fz, w11 = fy * fz;
-    const float w000 = gx * w00, w100 = fx * w00, w010 = gx * w10, w110 = fx * w10;
-    const float w001 = gx * w01, w101 = fx * w01, w011 = gx * w11, w111 = fx * w11;
-    c.x = w000 * v000.x;
-    c.y = w000 * v000.y;
-    c.z = w000 * v000.z;
-    c.w = w000 * v000.w;
-#define HH_ACC(W, V)              \
-    c.x = fmaf(W, V.x, c.x);      \
-    c.y = fmaf(W, V.y, c.y);      \
-    c.z = fmaf(W, V.z, c.z);      \
-    c.w = fmaf(W, V.w, c.w);
-    HH_ACC(w100, v100)
-    HH_ACC(w010, v010)
-    HH_ACC(w110, v110)
-    HH_ACC(w001, v001)
-    HH_ACC(w101, v101)
-    HH_ACC(w011, v011)
-    HH_ACC(w111, v111)
-#undef HH_ACC
+        // the standard 8-corner weights
+        const float4 v000 = __ldg(c00), v100 = __ldg(c00 + 2), v010 = __ldg(c10), v110 = __ldg(c10 + 2);
+        const float4 v001 = __ldg(c01), v101 = __ldg(c01 + 2), v011 = __ldg(c11), v111 = __ldg(c11 + 2);
+        const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
+        const float w00 = gy * gz, w10 = fy * gz, w01 = gy * fz, w11 = fy * fz;
+        const float w000 = gx * w00;
+        c.x = w000 * v000.x;
+        c.y = w000 * v000.y;
+        c.z = w000 * v000.z;
+        c.w = w000 * v000.w;
+        auto add = [&c](float w, const float4& v) {
+            c.x = fmaf(w, v.x, c.x);
+            c.y = fmaf(w, v.y, c.y);
+            c.z = fmaf(w, v.z, c.z);
+            c.w = fmaf(w, v.w, c.w);
+        };
+        add(fx * w00, v100);
+        add(gx * w10, v010);
+        add(fx * w10, v110);
+        add(gx * w01, v001);
+        add(fx * w01, v101);
+        add(gx * w11, v011);
+        add(fx * w11, v111);
     }
     // FP16 storage: the sample stays in code units (value / scale); the
     // power-of-two scales are applied downstream, where a product by them is
@@ -323,11 +333,12 @@ __device__ __forceinline__ bool fetch_nonzero(const VolArgs& A, const void* __re
     return true;
 }
 
-template <int STORAGE, bool CLAMP>
+template <int STORAGE, int ADDR, bool MASK, bool CLAMP>
 __device__ __forceinline__ Sample fetch(const VolArgs& A, const void* __restrict__ vol, float3 u,
                                         uint32_t& flags) {
     Sample s;
-    if (!fetch_nonzero<STORAGE, CLAMP>(A, vol, u, flags, s)) s.dn = s.gx = s.gy = s.gz = 0.0f;
+    if (!fetch_nonzero<STORAGE, ADDR, MASK, CLAMP>(A, vol, u, flags, s))
+        s.dn = s.gx = s.gy = s.gz = 0.0f;
     return s;
 }
 
@@ -517,11 +528,12 @@ __device__ __forceinline__ float3 perp_of(const Sample& s, float3 w, float s_n, 
     if (STORAGE != HH_STORE_FP32) gperp_norm *= s_g;
     return gp;
 }
-template <int STORAGE, bool CLAMP>
+template <int STORAGE, int ADDR, bool MASK, bool CLAMP>
 __device__ __forceinline__ float3 perp_rate(const VolArgs& A, const void* __restrict__ vol,
                                             float3 u, float3 w, float s_n, float s_g, float& n,
                                             float& gperp_norm, uint32_t& flags) {
-    return perp_of<STORAGE>(fetch<STORAGE, CLAMP>(A, vol, u, flags), w, s_n, s_g, n, gperp_norm);
+    return perp_of<STORAGE>(fetch<STORAGE, ADDR, MASK, CLAMP>(A, vol, u, flags), w, s_n, s_g, n,
+                            gperp_norm);
 }
 
 // Per-ray state of the march: primary direction w_ref, deflection d, biased
@@ -540,8 +552,8 @@ struct RayState {
 // 8-lane quarter of the warp covers a 4x2 pixel block, not a row of 8: a
 // 128-bit load is served a quarter-warp at a time, and the voxels of a 4x2
 // block of neighbouring rays form a 2x2 patch across the view, which falls on
-// four different micro-brick slots (L1 bank groups), where a row of 8 rays
-// would walk a line of voxels that alternates between two.
+// four different L1 bank groups, where a row of 8 rays would walk a line of
+// voxels that alternates between two.
 __device__ __forceinline__ void tile_pixel(int p, int tile_w_log2, int& x, int& y) {
     const int q = p >> 3;
     const int qx_log2 = tile_w_log2 - 2;  // quarters per tile row: 1, 2 or 4
@@ -582,7 +594,7 @@ __device__ __forceinline__ void ray_begin(const VolArgs& V, const float* __restr
 // One step of Eq. 16 (or RK4) with the Eq. 18 (or fixed) step length.
 // Returns true when the step leaves the box: then ep / ed hold the exit
 // point on the face and the new direction.
-template <int STORAGE, int STEPPER, bool ADAPTIVE>
+template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR, bool MASK>
 __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restrict__ vol, RayState& R,
                                          float3& ep, float3& ed) {
     const float B = V.bias;
@@ -594,23 +606,23 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
     if (STEPPER == HH_STEP_RK4) {
         float n1, gpn, n2, n3, n4, unused;
         const float3 w1 = wr + d;
-        const float3 gp1 = perp_rate<STORAGE, true>(V, vol, C, w1, R.sn, R.sg, n1, gpn, R.flags);
+        const float3 gp1 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, C, w1, R.sn, R.sg, n1, gpn, R.flags);
         ds = step_length<ADAPTIVE>(V, n1, gpn);
         const float hds = 0.5f * ds;
         const float3 k1 = (__fdividef(1.0f, n1) * gsc) * gp1;
         const float3 d2 = fma3(hds, k1, d);
         const float3 w2 = wr + d2;
-        const float3 gp2 = perp_rate<STORAGE, true>(V, vol, fma3(hds, w1, C), w2, R.sn, R.sg, n2,
+        const float3 gp2 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(hds, w1, C), w2, R.sn, R.sg, n2,
                                                     unused, R.flags);
         const float3 k2 = (__fdividef(1.0f, n2) * gsc) * gp2;
         const float3 d3 = fma3(hds, k2, d);
         const float3 w3 = wr + d3;
-        const float3 gp3 = perp_rate<STORAGE, true>(V, vol, fma3(hds, w2, C), w3, R.sn, R.sg, n3,
+        const float3 gp3 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(hds, w2, C), w3, R.sn, R.sg, n3,
                                                     unused, R.flags);
         const float3 k3 = (__fdividef(1.0f, n3) * gsc) * gp3;
         const float3 d4 = fma3(ds, k3, d);
         const float3 w4 = wr + d4;
-        const float3 gp4 = perp_rate<STORAGE, true>(V, vol, fma3(ds, w3, C), w4, R.sn, R.sg, n4,
+        const float3 gp4 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(ds, w3, C), w4, R.sn, R.sg, n4,
                                                     unused, R.flags);
         const float3 k4 = (__fdividef(1.0f, n4) * gsc) * gp4;
         // k1 + 2 (k2 + k3) + k4 (every k is a product: the adds are kept
@@ -626,7 +638,7 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
     } else {
         Sample smp;
         float3 d1;
-        if (fetch_nonzero<STORAGE, false>(V, vol, C, R.flags, smp)) {
+        if (fetch_nonzero<STORAGE, ADDR, MASK, false>(V, vol, C, R.flags, smp)) {
             float n, gpn;
             const float3 gp = perp_of<STORAGE>(smp, wr + d, R.sn, R.sg, n, gpn);
             ds = step_length<ADAPTIVE>(V, n, gpn);
@@ -669,6 +681,23 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
         return true;
     }
     return false;
+}
+
+// Marches a ray that entered the box until it leaves it or runs out of steps.
+// `sparse` (the same for every ray of the volume) picks the loop that tests the
+// free-corner mask or the one that does not.
+template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
+__device__ __forceinline__ void ray_march(const VolArgs& V, const void* __restrict__ vol,
+                                          unsigned sparse, RayState& R, float3& ep, float3& ed) {
+    if (sparse) {
+        while (R.k < V.max_steps &&
+               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, vol, R, ep, ed)) {
+        }
+    } else {
+        while (R.k < V.max_steps &&
+               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, vol, R, ep, ed)) {
+        }
+    }
 }
 
 // Display byte of a colour in [0, 1]: round-to-nearest-even of 255 v.
@@ -719,7 +748,7 @@ __device__ __forceinline__ void ray_end(const VolArgs& V, const ViewArgs& C, int
 
 // One view, one thread per pixel: a block of 128 threads covers 16x8 pixels,
 // each warp an 8x4 tile.
-template <int STORAGE, int STEPPER, bool ADAPTIVE>
+template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
 __global__ void __launch_bounds__(128, (STEPPER == HH_STEP_RK4) ? 6 : HH_MARCH_MIN_BLOCKS)
     march_kernel(const VolArgs V, const ViewArgs C) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -732,8 +761,7 @@ __global__ void __launch_bounds__(128, (STEPPER == HH_STEP_RK4) ? 6 : HH_MARCH_M
     float3 ep = C.eye, ed = C.eye;
     ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
     if (R.flags & HH_FLAG_HIT)
-        while (R.k < V.max_steps && !ray_step<STORAGE, STEPPER, ADAPTIVE>(V, V.vol, R, ep, ed)) {
-        }
+        ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, __ldg(V.sparse), R, ep, ed);
     ray_end(V, C, px, py, R, ep, ed);
 }
 
@@ -773,7 +801,7 @@ __device__ __forceinline__ void tile_of(int t, int n_views, const int* s_begin,
 // march them side by side on one SM, sharing its L1, and meet at a barrier
 // before the next group, as march_kernel's blocks do when they retire. The
 // per-ray arithmetic is march_kernel's.
-template <int STORAGE, int STEPPER, bool ADAPTIVE, bool REFILL>
+template <int STORAGE, int STEPPER, bool ADAPTIVE, bool REFILL, int ADDR>
 __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_MIN_BLOCKS)
     march_batch_kernel(const VolArgs V, const ViewArgs* __restrict__ views, int n_views,
                        int total_tiles, int tile_w, unsigned* __restrict__ counter,
@@ -786,6 +814,7 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     const int tile_w_log2 = tile_w == 16 ? 4 : (tile_w == 8 ? 3 : 2);
+    const unsigned sparse = __ldg(V.sparse);
     if (!REFILL) {
         __shared__ int s_group;  // first tile of the block's current group
         const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
@@ -816,8 +845,7 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
                 float3 ep = make_float3(0.0f, 0.0f, 0.0f), ed = ep;
                 ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
                 if (R.flags & HH_FLAG_HIT)
-                    while (R.k < V.max_steps && !ray_step<STORAGE, STEPPER, ADAPTIVE>(V, V.vol, R, ep, ed)) {
-                    }
+                    ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, sparse, R, ep, ed);
                 ray_end(V, C, px, py, R, ep, ed);
             }
         }
@@ -871,7 +899,10 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
             continue;
         }
         if (have) {
-            if (ray_step<STORAGE, STEPPER, ADAPTIVE>(V, V.vol, R, ep, ed) || R.k >= V.max_steps) {
+            const bool left =
+                sparse ? ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, V.vol, R, ep, ed)
+                       : ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, V.vol, R, ep, ed);
+            if (left || R.k >= V.max_steps) {
                 ray_end(V, views[vi], px, py, R, ep, ed);
                 have = false;
             }
@@ -940,6 +971,7 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
     int view_first = 0, view_end = 0;  // job-relative tiles of the view in C
     const void* jvol = nullptr;
     const float* jscales = nullptr;
+    unsigned jsparse = 0;
     int jview_begin = 0, jn_views = 0, jn_tiles = 0;
     unsigned t = 0;  // this warp's claimed tile of job j (valid while have_job == j)
     bool claimed_next = false;
@@ -1016,6 +1048,8 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
                 __ldcg(reinterpret_cast<const unsigned long long*>(&e->vol)));
             jscales = reinterpret_cast<const float*>(
                 __ldcg(reinterpret_cast<const unsigned long long*>(&e->scales)));
+            jsparse = __ldcg(reinterpret_cast<const unsigned*>(
+                __ldcg(reinterpret_cast<const unsigned long long*>(&e->sparse))));
             jview_begin = __ldcg(&e->view_begin);
             jn_views = __ldcg(&e->n_views);
             jn_tiles = __ldcg(&e->n_tiles);
@@ -1060,8 +1094,7 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
             float3 ep = make_float3(0.0f, 0.0f, 0.0f), ed = ep;
             ray_begin<ADAPTIVE>(V, jscales, C, px, py, R);
             if (R.flags & HH_FLAG_HIT)
-                while (R.k < V.max_steps && !ray_step<STORAGE, STEPPER, ADAPTIVE>(V, jvol, R, ep, ed)) {
-                }
+                ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>(V, jvol, jsparse, R, ep, ed);
             ray_end(V, C, px, py, R, ep, ed);
         }
         // count the tile (release: its outputs are ordered before the count,
@@ -1086,11 +1119,18 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
     }
 }
 
+// ADDR_BASE wherever the volume's byte offsets fit 32 bits (V.mask_off is the
+// end of its data).
+bool addr_any(const VolArgs& V) { return V.mask_off >= (1ull << 32); }
+
 template <int STORAGE, int STEPPER, bool ADAPTIVE>
 void launch_one(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
     const dim3 block(128);
     const dim3 grid((C.W + 15) / 16, (C.H + 7) / 8);
-    march_kernel<STORAGE, STEPPER, ADAPTIVE><<<grid, block, 0, s>>>(V, C);
+    if (addr_any(V))
+        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY><<<grid, block, 0, s>>>(V, C);
+    else
+        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_BASE><<<grid, block, 0, s>>>(V, C);
 }
 
 // Calls F<STORAGE, STEPPER, ADAPTIVE>::run(args...) for the runtime choice.
@@ -1114,19 +1154,26 @@ struct SingleLaunch {
     }
 };
 
-// refill_min >= 32 runs the tile-at-a-time instantiation (REFILL = false).
+// The batch kernel of a launch: refill_min >= 32 runs the tile-at-a-time
+// instantiation (REFILL = false).
+template <int ST, int SP, bool AD>
+auto batch_kernel(bool any, int refill_min) {
+    if (refill_min >= 32)
+        return any ? march_batch_kernel<ST, SP, AD, false, ADDR_ANY>
+                   : march_batch_kernel<ST, SP, AD, false, ADDR_BASE>;
+    return any ? march_batch_kernel<ST, SP, AD, true, ADDR_ANY>
+               : march_batch_kernel<ST, SP, AD, true, ADDR_BASE>;
+}
+
 template <int ST, int SP, bool AD>
 struct BatchLaunch {
     static void run(const VolArgs& V, const ViewArgs* views, int n_views, int total_tiles,
                     int tile_w, unsigned* counter, int refill_min, const uint2* order, int group,
                     int blocks, int threads, cudaStream_t s) {
         const size_t smem = (n_views + 1) * sizeof(int);
-        if (refill_min >= 32)
-            march_batch_kernel<ST, SP, AD, false><<<blocks, threads, smem, s>>>(
-                V, views, n_views, total_tiles, tile_w, counter, refill_min, order, group);
-        else
-            march_batch_kernel<ST, SP, AD, true><<<blocks, threads, smem, s>>>(
-                V, views, n_views, total_tiles, tile_w, counter, refill_min, order, 0);
+        batch_kernel<ST, SP, AD>(addr_any(V), refill_min)<<<blocks, threads, smem, s>>>(
+            V, views, n_views, total_tiles, tile_w, counter, refill_min, order,
+            refill_min >= 32 ? group : 0);
     }
 };
 
@@ -1149,13 +1196,9 @@ struct WorkerOccupancy {
 
 template <int ST, int SP, bool AD>
 struct BatchOccupancy {
-    static void run(int threads, size_t smem, int refill_min, int* blocks_per_sm) {
-        if (refill_min >= 32)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                blocks_per_sm, march_batch_kernel<ST, SP, AD, false>, threads, smem);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                blocks_per_sm, march_batch_kernel<ST, SP, AD, true>, threads, smem);
+    static void run(int threads, size_t smem, bool any, int refill_min, int* blocks_per_sm) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            blocks_per_sm, batch_kernel<ST, SP, AD>(any, refill_min), threads, smem);
     }
 };
 
@@ -1166,11 +1209,13 @@ VolArgs make_vol_args(const hh_volume_s* vol, const hh_step_params& P, const hh_
     A.nx = vol->nx;
     A.ny = vol->ny;
     A.nz = vol->nz;
-    A.bx = vol->bx;
-    A.bxy = vol->bxy;
-    A.by8 = vol->bx * 8u;
-    A.bz8 = vol->bxy * 8u;
-    A.mask_off = vol->bytes;
+    A.sparse = vol->sparse_dev;
+    A.row = vol->row;
+    A.half_pair = vol->pair / 2;
+    const unsigned voxel_bytes = vol->storage == HH_STORE_FP32 ? 16u : 8u;
+    A.row_bytes = vol->row * voxel_bytes;
+    A.up_bytes = (vol->pair - 2u) * voxel_bytes;
+    A.mask_off = vol->mask_off;
     // bias: a power of two B with B >= 2 * step and B >= extent + step + 1, so
     // positions in [-step, extent + step] keep hi in [B/2, 2B - 1] and both
     // hi - B and hi - (B - 1/2) are exact (Sterbenz)
@@ -1240,7 +1285,7 @@ ViewArgs make_view_args(const hh_camera& cam, const hh_view_out& out, int tile_w
 
 cudaError_t launch_trace(const hh_volume_s* vol, const hh_camera& cam, const hh_step_params& P,
                          const hh_background& bg, const hh_view_out& out, cudaStream_t s) {
-    if (vol->layout != HH_LAYOUT_BRICK2) return cudaErrorInvalidValue;
+    if (vol->layout != HH_LAYOUT_ZPAIR) return cudaErrorInvalidValue;
     const VolArgs V = make_vol_args(vol, P, bg);
     const ViewArgs C = make_view_args(cam, out, 8);
     dispatch<SingleLaunch>(vol->storage, P.stepper, P.adaptive, V, C, s);
@@ -1277,7 +1322,7 @@ int serve_worker_blocks_per_sm(int storage, int stepper, int adaptive, int threa
 cudaError_t launch_serve_worker(const hh_volume_s* like, const hh_step_params& P,
                                 const hh_background& bg, const ServeWorkerArgs& W, int blocks,
                                 int threads, cudaStream_t s) {
-    if (like->layout != HH_LAYOUT_BRICK2) return cudaErrorInvalidValue;
+    if (like->layout != HH_LAYOUT_ZPAIR) return cudaErrorInvalidValue;
     const VolArgs V = make_vol_args(like, P, bg);
     dispatch<WorkerLaunch>(like->storage, P.stepper, P.adaptive, V, W, blocks, threads, s);
     count_launch();
@@ -1394,7 +1439,7 @@ int resident_blocks(hh_batch b, int threads, int refill_min) {
     int bps = 0;
     const size_t smem = (b->cams.size() + 1) * sizeof(int);
     hh::dispatch<hh::BatchOccupancy>(b->vol->storage, b->params.stepper, b->params.adaptive,
-                                     threads, smem, refill_min, &bps);
+                                     threads, smem, b->vol->mask_off >= (1ull << 32), refill_min, &bps);
     return std::max(bps, 1);
 }
 

@@ -244,6 +244,7 @@ hh_status hh_server_s::publish(Request& r) {
     hh::ServeJob& e = jobs_host[j];
     e.vol = vol->data;
     e.scales = vol->scales_dev;
+    e.sparse = vol->sparse_dev;
     e.view_begin = next_view;
     e.n_views = n;
     e.n_tiles = tiles;
@@ -580,8 +581,8 @@ hh_status hh_serve_set_config(hh_server S, const hh_batch_config* cfg) {
 
 hh_status hh_serve_put_volume(hh_server S, int64_t frame_id, hh_volume vol) {
     if (!S || !vol) return hh::fail(HH_ERR_INVALID_ARG, "server or volume is NULL");
-    if (vol->layout != HH_LAYOUT_BRICK2)
-        return hh::fail(HH_ERR_INVALID_ARG, "the volume is not a marchable (BRICK2) volume");
+    if (vol->layout != HH_LAYOUT_ZPAIR)
+        return hh::fail(HH_ERR_INVALID_ARG, "the volume is not a marchable (ZPAIR) volume");
     std::lock_guard<std::mutex> lock(S->mu);
     if (S->frame_users.count(frame_id))
         return hh::fail(HH_ERR_BUSY, "frame %lld is being rendered", static_cast<long long>(frame_id));
