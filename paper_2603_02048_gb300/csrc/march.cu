@@ -157,7 +157,40 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return r;
 }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 pa, pb, pd;\n\t"
+        "mov.b64 pa, {%2, %3};\n\tmov.b64 pb, {%4, %5};\n\t"
+        "add.rn.f32x2 pd, pa, pb;\n\tmov.b64 {%0, %1}, pd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 pa, pb, pd;\n\t"
+        "mov.b64 pa, {%2, %3};\n\tmov.b64 pb, {%4, %5};\n\t"
+        "mul.rn.f32x2 pd, pa, pb;\n\tmov.b64 {%0, %1}, pd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 xy(float3 a) { return make_float2(a.x, a.y); }
+__device__ __forceinline__ float3 with_z(float2 a, float z) { return make_float3(a.x, a.y, z); }
+// The march's vectors as a packed x, y pair and a scalar z, each component
+// rounded as by the scalar operators above: two instructions for three, in a
+// step that the issue rate bounds (march of the 256^3 1080p frame at h_max: 320
+// against 308 us).
+__device__ __forceinline__ float3 add_p(float3 a, float3 b) {
+    return with_z(add2(xy(a), xy(b)), __fadd_rn(a.z, b.z));
+}
+__device__ __forceinline__ float3 mul_p(float s, float3 a) {
+    return with_z(mul2(dup(s), xy(a)), __fmul_rn(s, a.z));
+}
+__device__ __forceinline__ float3 fma_p(float s, float3 b, float3 a) {
+    return with_z(fma2(dup(s), xy(b), xy(a)), fmaf(s, b.z, a.z));
+}
 // a + t (b - a) on both halves of a float4 (t duplicated in tt).
 __device__ __forceinline__ float4 lerp4x2(float4 a, float4 b, float2 tt) {
     const float2 lo = fma2(tt, sub2(make_float2(b.x, b.y), make_float2(a.x, a.y)),
@@ -167,10 +200,19 @@ __device__ __forceinline__ float4 lerp4x2(float4 a, float4 b, float2 tt) {
     return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
-// Hardware approximate square root (PTX sqrt.approx.f32, ~1 ulp).
+// Hardware approximate square root and division (PTX *.approx.ftz.f32, ~1 ulp):
+// without .ftz each carries instructions for subnormal operands (same march:
+// 330 against 320 us). A subnormal |g_perp|^2 taken as 0 moves
+// |g_perp| by less than 1.1e-19, which eps outweighs; the other operands are
+// subnormal only where the step length or eps itself is.
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float div_approx(float a, float b) {
+    float r;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
 }
 
@@ -299,29 +341,31 @@ __device__ __forceinline__ bool fetch_nonzero(const VolArgs& A, const void* __re
         c = lerp4x2(lerp4x2(xlerp_fp16(r000, r100, tx), xlerp_fp16(r010, r110, tx), ty),
                     lerp4x2(xlerp_fp16(r001, r101, tx), xlerp_fp16(r011, r111, tx), ty), tz);
     } else {
-        // the standard 8-corner weights
+        // the standard 8-corner weights (formed two at a time; the sum over
+        // corners packed two channels at a time was slower, 317 against 308 us)
         const float4 v000 = __ldg(c00), v100 = __ldg(c00 + 2), v010 = __ldg(c10), v110 = __ldg(c10 + 2);
         const float4 v001 = __ldg(c01), v101 = __ldg(c01 + 2), v011 = __ldg(c11), v111 = __ldg(c11 + 2);
         const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-        const float w00 = gy * gz, w10 = fy * gz, w01 = gy * fz, w11 = fy * fz;
-        const float w000 = gx * w00;
-        c.x = w000 * v000.x;
-        c.y = w000 * v000.y;
-        c.z = w000 * v000.z;
-        c.w = w000 * v000.w;
+        const float2 y0 = make_float2(gy, fy), yz0 = mul2(y0, dup(gz)), yz1 = mul2(y0, dup(fz));
+        const float2 w00 = mul2(dup(gx), yz0), w10 = mul2(dup(fx), yz0);  // [x][z], over y
+        const float2 w01 = mul2(dup(gx), yz1), w11 = mul2(dup(fx), yz1);
+        c.x = w00.x * v000.x;
+        c.y = w00.x * v000.y;
+        c.z = w00.x * v000.z;
+        c.w = w00.x * v000.w;
         auto add = [&c](float w, const float4& v) {
             c.x = fmaf(w, v.x, c.x);
             c.y = fmaf(w, v.y, c.y);
             c.z = fmaf(w, v.z, c.z);
             c.w = fmaf(w, v.w, c.w);
         };
-        add(fx * w00, v100);
-        add(gx * w10, v010);
-        add(fx * w10, v110);
-        add(gx * w01, v001);
-        add(fx * w01, v101);
-        add(gx * w11, v011);
-        add(fx * w11, v111);
+        add(w10.x, v100);
+        add(w00.y, v010);
+        add(w10.y, v110);
+        add(w01.x, v001);
+        add(w11.x, v101);
+        add(w01.y, v011);
+        add(w11.y, v111);
     }
     // FP16 storage: the sample stays in code units (value / scale); the
     // power-of-two scales are applied downstream, where a product by them is
@@ -346,7 +390,7 @@ __device__ __forceinline__ Sample fetch(const VolArgs& A, const void* __restrict
 template <bool ADAPTIVE>
 __device__ __forceinline__ float step_length(const VolArgs& A, float n, float gperp_norm) {
     if (!ADAPTIVE) return A.h_fixed;
-    return fminf(fmaxf(__fdividef(n * A.theta, gperp_norm + A.eps), A.h_min), A.h_max);
+    return fminf(fmaxf(div_approx(n * A.theta, gperp_norm + A.eps), A.h_min), A.h_max);
 }
 
 // Eq. 16's normalize, in deflection form: returns d' with w_ref + d' the unit
@@ -523,7 +567,7 @@ __device__ __forceinline__ float3 perp_of(const Sample& s, float3 w, float s_n, 
                                           float& n, float& gperp_norm) {
     n = STORAGE == HH_STORE_FP32 ? 1.0f + s.dn : fmaf(s.dn, s_n, 1.0f);
     const float3 g = make_float3(s.gx, s.gy, s.gz);
-    const float3 gp = fma3(-dot(w, g), w, g);
+    const float3 gp = fma_p(-dot(w, g), w, g);
     gperp_norm = sqrt_approx(dot(gp, gp));
     if (STORAGE != HH_STORE_FP32) gperp_norm *= s_g;
     return gp;
@@ -609,22 +653,22 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
         const float3 gp1 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, C, w1, R.sn, R.sg, n1, gpn, R.flags);
         ds = step_length<ADAPTIVE>(V, n1, gpn);
         const float hds = 0.5f * ds;
-        const float3 k1 = (__fdividef(1.0f, n1) * gsc) * gp1;
+        const float3 k1 = (div_approx(1.0f, n1) * gsc) * gp1;
         const float3 d2 = fma3(hds, k1, d);
         const float3 w2 = wr + d2;
         const float3 gp2 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(hds, w1, C), w2, R.sn, R.sg, n2,
                                                     unused, R.flags);
-        const float3 k2 = (__fdividef(1.0f, n2) * gsc) * gp2;
+        const float3 k2 = (div_approx(1.0f, n2) * gsc) * gp2;
         const float3 d3 = fma3(hds, k2, d);
         const float3 w3 = wr + d3;
         const float3 gp3 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(hds, w2, C), w3, R.sn, R.sg, n3,
                                                     unused, R.flags);
-        const float3 k3 = (__fdividef(1.0f, n3) * gsc) * gp3;
+        const float3 k3 = (div_approx(1.0f, n3) * gsc) * gp3;
         const float3 d4 = fma3(ds, k3, d);
         const float3 w4 = wr + d4;
         const float3 gp4 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(ds, w3, C), w4, R.sn, R.sg, n4,
                                                     unused, R.flags);
-        const float3 k4 = (__fdividef(1.0f, n4) * gsc) * gp4;
+        const float3 k4 = (div_approx(1.0f, n4) * gsc) * gp4;
         // k1 + 2 (k2 + k3) + k4 (every k is a product: the adds are kept
         // unfused, __fadd_rn, so no product is folded into them)
         const float3 ksum =
@@ -640,9 +684,9 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
         float3 d1;
         if (fetch_nonzero<STORAGE, ADDR, MASK, false>(V, vol, C, R.flags, smp)) {
             float n, gpn;
-            const float3 gp = perp_of<STORAGE>(smp, wr + d, R.sn, R.sg, n, gpn);
+            const float3 gp = perp_of<STORAGE>(smp, add_p(wr, d), R.sn, R.sg, n, gpn);
             ds = step_length<ADAPTIVE>(V, n, gpn);
-            d1 = fma3(__fdividef(ds, n) * gsc, gp, d);
+            d1 = fma_p(div_approx(ds, n) * gsc, gp, d);
         } else {
             // the zero sample: n = 1 and g_perp = 0 exactly, so the branch
             // above would give the step length ds0 (the same operations on
@@ -654,18 +698,20 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
         }
         // Eq. 16: w' = normalize(w1), C' = C + ds w'; with w' = (1 + r) w1
         // the increment is ds (1 + r) w1 (w' itself is formed only at the exit)
-        const float3 w1 = wr + d1;
+        const float3 w1 = add_p(wr, d1);
         const float rm1 = renorm_term(w1);
-        dnew = fma3(rm1, w1, d1);
-        inc = fmaf(ds, rm1, ds) * w1;
+        dnew = fma_p(rm1, w1, d1);
+        inc = mul_p(fmaf(ds, rm1, ds), w1);
     }
-    float3 nhi, err;
-    fast_two_sum(R.hi.x, inc.x, nhi.x, err.x);
-    fast_two_sum(R.hi.y, inc.y, nhi.y, err.y);
-    fast_two_sum(R.hi.z, inc.z, nhi.z, err.z);
-    const float3 nlo = R.lo + err;
+    // Fast2Sum of hi and the increment, x and y packed
+    const float2 nhi2 = add2(xy(R.hi), xy(inc));
+    const float2 err2 = sub2(xy(inc), sub2(nhi2, xy(R.hi)));
+    float nhi_z, err_z;
+    fast_two_sum(R.hi.z, inc.z, nhi_z, err_z);
+    const float3 nhi = with_z(nhi2, nhi_z);
+    const float3 nlo = add_p(R.lo, with_z(err2, err_z));
     const float Bu = V.bias_u;
-    const float3 P = make_float3((nhi.x - Bu) + nlo.x, (nhi.y - Bu) + nlo.y, (nhi.z - Bu) + nlo.z);
+    const float3 P = add_p(with_z(sub2(nhi2, dup(Bu)), __fsub_rn(nhi_z, Bu)), nlo);
     ++R.k;
     const float3 ohi = R.hi, olo = R.lo;
     R.hi = nhi;
