@@ -2,14 +2,12 @@
 // rho(x_v) = sum_p m_p W(|x_v - x_p|, h) at voxel centres, W the M4 cubic
 // spline with support 2h.
 //
-// Two kernels: splat_box8_kernel for supports of at most 8 voxels per axis
-// (2h <= 4, the paper's h = 2), described where it is defined, and
-// splat_warp_kernel for wider ones. Both put four particles on a warp,
-// eight lanes each, so that a warp's reductions at one (y, z) row cover four
-// 8-float runs (four 32-byte sectors, one per particle) and compile to
-// fire-and-forget reductions in L2, and the per-particle set-up is shared by
-// the four particles' lanes (against one particle per warp this took 12 %
-// off the build; eight per warp, half-sector reductions, was slower again).
+// Two kernels: splat_box_kernel for supports of at most 16 voxels per axis (2h
+// <= 8, the paper's h = 2 among them), described where it is defined, and
+// splat_warp_kernel for wider ones, four particles a warp, eight lanes each, so
+// that a warp's reductions at one (y, z) row cover four 8-float runs (four
+// 32-byte sectors, one per particle) and compile to fire-and-forget reductions
+// in L2, and the per-particle set-up is shared by the four particles' lanes.
 //
 // splat_warp_kernel: a lane owns an (x, y) column of its particle's
 // footprint (the voxels whose centres lie within 2h on every axis), the
@@ -19,6 +17,7 @@
 // (grids hold fewer than 2^31 voxels). The kernel is evaluated in r with the
 // particle's mass folded into its coefficients.
 #include <algorithm>
+#include <cmath>
 
 #include "hh_internal.h"
 
@@ -29,7 +28,8 @@ namespace {
 // W = norm (1 - 3/2 q^2 + 3/4 q^3) on q = r/h < 1, norm (2 - q)^3 / 4 on
 // [1, 2), norm = 1 / (pi h^3); in r: m W = mn + r^2 (c2 + c3 r) for r < h and
 // d (2h - r)^3 beyond, mn = m norm, c2 = -3/2 mn / h^2, c3 = 3/4 mn / h^3,
-// d = mn / (4 h^3). Both pieces are evaluated and selected (no divergence).
+// d = mn / (4 h^3). Both pieces are evaluated and selected (no divergence). For r
+// below 2h.
 struct M4Coef {
     float mn, c2, c3, d, h, two_h;
 };
@@ -48,7 +48,7 @@ __device__ __forceinline__ M4Coef m4_coef(float m, float h, float inv_h, float n
 
 __device__ __forceinline__ float m4_mass(const M4Coef& c, float r2, float r) {
     const float inner = fmaf(r2, fmaf(c.c3, r, c.c2), c.mn);
-    const float t = fmaxf(c.two_h - r, 0.0f);
+    const float t = c.two_h - r;
     const float outer = c.d * (t * t * t);
     return r < c.h ? inner : outer;
 }
@@ -69,7 +69,7 @@ __device__ __forceinline__ void footprint(float x, float reach, int n, int& lo, 
     hi = min(n - 1, (int)floorf(b));
 }
 
-constexpr int kParticlesPerWarp = 4;
+constexpr int kParticlesPerWarp = 4;  // of splat_warp_kernel
 
 template <int PPW>  // particles per warp: 32 / PPW lanes each
 __global__ void __launch_bounds__(256) splat_warp_kernel(const float4* __restrict__ parts,
@@ -138,13 +138,14 @@ __device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t b, uint64_t c)
     return r;
 }
 
-// First of the 8 voxel slots along one axis that cover every voxel centre
-// within `reach` (<= 4) of x: the smallest k with k + 1/2 > x - reach,
-// clamped to [-8, n] so that the slots' indices stay small (slots outside
+// First of the N voxel slots along one axis that cover every voxel centre
+// within `reach` (<= N / 2) of x: the smallest k with k + 1/2 > x - reach,
+// clamped to [-N, n] so that the slots' indices stay small (slots outside
 // [0, n) are masked by their distance; NaN converts to 0 and is masked the
 // same way).
-__device__ __forceinline__ int box8_start(float x, float reach, int n) {
-    const float a = fminf(fmaxf(x - reach - 0.5f, -9.0f), static_cast<float>(n));
+template <int N>
+__device__ __forceinline__ int box_start(float x, float reach, int n) {
+    const float a = fminf(fmaxf(x - reach - 0.5f, -(N + 1.0f)), static_cast<float>(n));
     return __float2int_rd(a) + 1;
 }
 
@@ -154,60 +155,93 @@ __device__ __forceinline__ float dist_or_inf(int k, int n, float x) {
     return (k >= 0 && k < n) ? (static_cast<float>(k) + 0.5f) - x : __int_as_float(0x7f800000);
 }
 
-// The splat for kernel radii 2h <= 4 voxels (the paper's h = 2 among them):
-// every particle's support fits an 8 x 8 x 8 box of voxel slots. Four
-// particles per warp, eight lanes each on the box's x slots; a lane walks its
-// 8 y rows and 8 z slots fully unrolled. Slots outside the grid get an
-// infinite distance, so no index test is needed per slot, and a slot adds
-// its mass only where it lies inside the support (a predicated reduction, no
-// branch). The kernel is evaluated in the branch-free form
-// m W = m norm (2 t^3 - u^3), t = 1 - r/2h, u = max(1 - r/h, 0), equal to the
-// two-piece M4 on [0, 2h): 2 t^3 = (2 - q)^3 / 4 and u^3 = (1 - q)^3 for
-// q = r/h < 1. Against splat_warp_kernel (per-column and per-voxel branches,
-// the footprint walked in loops) this issues a third fewer instructions and
-// the 256^3 plume's splat drops from 120 to 91 us; packed FP32x2 arithmetic
-// for slot pairs issues fewer still but is no faster, the L2 reductions now
-// setting the pace.
-template <int PPW>
-__global__ void __launch_bounds__(256) splat_box8_kernel(const float4* __restrict__ parts,
-                                                         int64_t n, int nx, int ny, int nz,
-                                                         float reach, float inv_2h, float inv_h,
-                                                         float norm, float* __restrict__ rho) {
-    constexpr int LPP = 32 / PPW;
-    static_assert(LPP == 8, "eight lanes per particle: one per x slot");
-    const int lane = threadIdx.x & 31;
-    const int64_t p =
-        ((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * PPW + lane / LPP;
+// The splat for kernel radii 2h <= N / 2 voxels: every particle's support fits
+// an N x N x N box of voxel slots. A particle has LPP lanes of a warp, dealt to
+// the N x N columns of its box LPP at a time, x fastest, and a lane walks its
+// column's N z slots fully unrolled. Slots outside the grid get an infinite
+// distance, so no index test is needed per slot, and a slot adds its mass only
+// where it lies inside the support (a predicated reduction, no branch). Where
+// h is a power of two, so that dividing by it is exact (UNIT; also below h = 1/2),
+// the M4 is evaluated as m norm (2 t^3 - u^3), t = 1 - r / 2h, u = sat(1 - r / h),
+// equal to its two pieces on [0, 2h); else by pieces (m4_mass), as fast and
+// without the rounding of 1 / h in every distance.
+// What bounds it: the L2 reductions (0.7-0.8 T float additions a second) and
+// the issue rate, together at N = 8 (83 % issue, 262,144 particles on 256^3 in
+// 90 us). Packed FP32x2 arithmetic issues fewer instructions but is no faster;
+// vector reductions (.v2, .v4 on aligned x runs, or on a bricked density) are
+// slower there (111-184 us). 60,011 particles on 161x118x97, with the
+// density's memset, against splat_warp_kernel (N <= 8: against the 8-slot box):
+//   h     1 (N = 4)  1.5 (6)  2.5 (10)  3 (12)  4 (16)
+//   before   27        27        87       137     228 us
+//   now      16        22        56        75     149 us
+// The split of the lanes matters little (N = 12: 84 us with 8 lanes, 78 with
+// 16, 92 with rows of 12 in 16 lanes).
+template <int N, int LPP, bool UNIT>
+__global__ void __launch_bounds__(256) splat_box_kernel(const float4* __restrict__ parts,
+                                                        int64_t n, int nx, int ny, int nz,
+                                                        float h, float inv_h, float norm,
+                                                        float* __restrict__ rho) {
+    const int lane = threadIdx.x & 31, sl = lane % LPP;
+    const int64_t p = ((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) *
+                          (32 / LPP) + lane / LPP;
     if (p >= n) return;
     const float4 q = __ldg(parts + p);
-    const int sx = box8_start(q.x, reach, nx), sy = box8_start(q.y, reach, ny),
-              sz = box8_start(q.z, reach, nz);
-    const int i = sx + (lane % LPP);
-    const float dx = dist_or_inf(i, nx, q.x);
-    const float dx2 = dx * dx;
-    float dz[8];
+    const float reach = 2.0f * h;
+    const float inv_2h = 0.5f * inv_h;
+    const int sx = box_start<N>(q.x, reach, nx), sy = box_start<N>(q.y, reach, ny),
+              sz = box_start<N>(q.z, reach, nz);
+    float dz[N];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) dz[k] = dist_or_inf(sz + k, nz, q.z);
+    for (int k = 0; k < N; ++k) dz[k] = dist_or_inf(sz + k, nz, q.z);
     const float mn = q.w * norm, c_t = 2.0f * mn, c_u = -mn;
+    const M4Coef cf = m4_coef(q.w, h, inv_h, norm);
     const uint64_t row_b = static_cast<uint64_t>(nx) * sizeof(float);
     // a plane is at most 16384^2 floats (1 GiB): its byte size fits 32 bits
     const uint32_t plane_b = static_cast<uint32_t>(row_b * static_cast<uint64_t>(ny));
-    // byte address of slot (i, sy, sz); unsigned arithmetic, formed for
-    // masked slots too but never dereferenced there
-    uint64_t row = reinterpret_cast<uint64_t>(rho) +
-                   static_cast<uint64_t>((static_cast<int64_t>(sz) * ny + sy) * nx + i) *
+    int cx = sl % N, cy = sl / N;  // this lane's column of the box
+    float dx = dist_or_inf(sx + cx, nx, q.x);
+    float dx2 = dx * dx;
+    // byte address of slot (sx + cx, sy + cy, sz); unsigned arithmetic, formed
+    // for masked slots too but never dereferenced there
+    uint64_t col = reinterpret_cast<uint64_t>(rho) +
+                   static_cast<uint64_t>((static_cast<int64_t>(sz) * ny + sy + cy) * nx + sx + cx) *
                        sizeof(float);
-#pragma unroll
-    for (int j = 0; j < 8; ++j, row += row_b) {
-        const float dy = dist_or_inf(sy + j, ny, q.y);
+    constexpr int kPasses = (N * N + LPP - 1) / LPP;
+    constexpr bool kTail = N * N % LPP != 0;  // columns past the last are masked
+#pragma unroll(N == 8 ? 8 : 1)
+    for (int m = 0; m < kPasses; ++m) {
+        const float dy = !kTail || cy < N ? dist_or_inf(sy + cy, ny, q.y)
+                                          : __int_as_float(0x7f800000);
         const float dxy2 = fmaf(dy, dy, dx2);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float r = sqrt_approx_ftz(fmaf(dz[k], dz[k], dxy2));
-            const float t = fmaf(r, -inv_2h, 1.0f);
-            const float u = __saturatef(fmaf(r, -inv_h, 1.0f));
-            const float w = fmaf(t * t * t, c_t, (u * u * u) * c_u);
-            red_add_if_positive(t, mad_wide(plane_b, k, row), w);
+        for (int k = 0; k < N; ++k) {
+            const float r2 = fmaf(dz[k], dz[k], dxy2), r = sqrt_approx_ftz(r2);
+            float t, w;
+            if (UNIT) {
+                t = fmaf(r, -inv_2h, 1.0f);
+                const float u = __saturatef(fmaf(r, -inv_h, 1.0f));
+                w = fmaf(t * t * t, c_t, (u * u * u) * c_u);
+            } else {
+                t = reach - r;
+                w = m4_mass(cf, r2, r);
+            }
+            red_add_if_positive(t, mad_wide(plane_b, k, col), w);
+        }
+        if (N == LPP) {  // the same column of the next row
+            ++cy;
+            col += row_b;
+        } else {  // LPP columns on
+            constexpr int kRows = LPP / N;  // whole rows in LPP columns
+            cx += LPP - kRows * N;
+            cy += kRows;
+            col += kRows * row_b + (LPP - kRows * N) * sizeof(float);
+            if (cx >= N) {
+                cx -= N;
+                ++cy;
+                col += row_b - N * sizeof(float);
+            }
+            dx = dist_or_inf(sx + cx, nx, q.x);
+            dx2 = dx * dx;
         }
     }
 }
@@ -359,17 +393,33 @@ cudaError_t launch_splat(const float4* xyzm, int64_t n, int nx, int ny, int nz, 
     if (e != cudaSuccess) return e;
     if (n == 0) return cudaSuccess;
     const int threads = 256;
-    const int64_t warps = (n + kParticlesPerWarp - 1) / kParticlesPerWarp;
-    const int64_t blocks = (warps * 32 + threads - 1) / threads;
+    auto blocks = [&](int ppw) {  // of warps with ppw particles each
+        return static_cast<unsigned>(((n + ppw - 1) / ppw * 32 + threads - 1) / threads);
+    };
     const double hd = h;
+    const float inv_h = static_cast<float>(1.0 / hd);
     const float norm = static_cast<float>(1.0 / (3.14159265358979323846 * hd * hd * hd));
-    if (2.0 * hd <= 4.0)
-        splat_box8_kernel<kParticlesPerWarp><<<static_cast<unsigned>(blocks), threads, 0, s>>>(
-            xyzm, n, nx, ny, nz, 2.0f * h, static_cast<float>(0.5 / hd),
-            static_cast<float>(1.0 / hd), norm, rho);
+    int e2 = 0;
+    const bool unit = hd < 0.5 || std::frexp(hd, &e2) == 0.5;
+    auto box = [&](auto kernel, int lanes) {
+        kernel<<<blocks(32 / lanes), threads, 0, s>>>(xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
+    };
+    // the smallest box that holds the support (4h slots an axis)
+    if (hd <= 1.0)
+        box(unit ? splat_box_kernel<4, 4, true> : splat_box_kernel<4, 4, false>, 4);
+    else if (hd <= 1.5)
+        box(splat_box_kernel<6, 8, false>, 8);
+    else if (hd <= 2.0)
+        box(unit ? splat_box_kernel<8, 8, true> : splat_box_kernel<8, 8, false>, 8);
+    else if (hd <= 2.5)
+        box(splat_box_kernel<10, 8, false>, 8);
+    else if (hd <= 3.0)
+        box(splat_box_kernel<12, 16, false>, 16);
+    else if (hd <= 4.0)
+        box(splat_box_kernel<16, 16, false>, 16);
     else
-        splat_warp_kernel<kParticlesPerWarp><<<static_cast<unsigned>(blocks), threads, 0, s>>>(
-            xyzm, n, nx, ny, nz, h, static_cast<float>(1.0 / hd), norm, rho);
+        splat_warp_kernel<kParticlesPerWarp><<<blocks(kParticlesPerWarp), threads, 0, s>>>(
+            xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
     count_launch();
     return cudaGetLastError();
 }
