@@ -52,14 +52,21 @@ namespace {
 
 constexpr float kPi = 3.14159265358979323846f;
 
-// Resident 128-thread blocks per SM the Eq. 16 march kernels are compiled
-// for: 8 leaves 64 registers per thread (measured fastest; 10 or 12 spill).
-#define HH_MARCH_MIN_BLOCKS 8
-// Resident 256-thread blocks per SM of the persistent batched kernel (its
-// refill state needs registers beyond the single-view kernel's).
-#ifndef HH_BATCH_MIN_BLOCKS
-#define HH_BATCH_MIN_BLOCKS 3
-#endif
+// Resident 128-thread blocks per SM the single-view march kernels are compiled
+// for: 8 leaves 64 registers a thread (Eq. 16; 9 or 10 measured the same, or
+// slower where they spill), 6 leaves 80 (RK4).
+constexpr int march_blocks(int stepper) { return stepper == HH_STEP_RK4 ? 6 : 8; }
+// Resident 256-thread blocks per SM of the persistent batched kernel. More
+// warps hide more of the L2 latency as long as the step does not spill. Tile at
+// a time, FP16: 5 blocks (48 registers) against 4, 8 views of the 256^3 volume
+// 1085 against 1088 us (views in turn: 1148 against 1195), 32 views of the 512^3
+// one 9.34 against 9.77 ms. FP32, whose eight corners take twice the
+// registers: 4 blocks (64) against 3 and 5, 8 views 1171 against 1239 and 1367
+// us. RK4 and the refill state need more registers.
+constexpr int batch_blocks(int storage, int stepper, bool refill) {
+    if (stepper == HH_STEP_RK4 || refill) return 3;
+    return storage == HH_STORE_FP32 ? 4 : 5;
+}
 
 // Volume-side arguments of a launch (shared by every view).
 struct VolArgs {
@@ -77,13 +84,14 @@ struct VolArgs {
     int max_steps;
     const uint8_t* bg;
     int bgW, bgH;
+    float bg_u, bg_v;   // texels per radian: bgW / 2 pi, bgH / pi
     int n_planes;
     hh_plane planes[HH_MAX_PLANES];
 };
 
 // View-side arguments: the camera, the caller's output buffers and the
 // view's place in a batch's tile list.
-struct ViewArgs {
+struct alignas(16) ViewArgs {
     float3 eye;
     float3 f, r, u;    // camera basis: forward, right, up (computed on the host in FP64)
     float a0, b0, s;   // pixel (x, y) -> a = a0 + (x + 1/2) s, b = b0 - (y + 1/2) s
@@ -219,7 +227,8 @@ __device__ __forceinline__ float div_approx(float a, float b) {
 // Lattice cell and weight along one axis from the lattice coordinate u =
 // position + 1/2, the halo coordinate of the ZPAIR layout (the centre of
 // grid voxel i at u = i + 1; the march carries u, not the position):
-// i0 = floor(u), f = u - i0. A position in [0, n] has u in [0.5, n + 0.5], so
+// i0 = floor(u), f = u - i0 (both from u itself: an index taken from the rounded
+// value would wait for it; march of the 256^3 frame 309 against 305 us). A position in [0, n] has u in [0.5, n + 0.5], so
 // both corners i0, i0 + 1 lie in the padded axis [0, n + 1], and the halo
 // copies make this the sample with the lattice coordinate clamped to the
 // voxel centres. The Euler march samples only accepted points, which lie in
@@ -228,9 +237,8 @@ __device__ __forceinline__ float div_approx(float a, float b) {
 template <bool CLAMP>
 __device__ __forceinline__ void axis_cell(float u, int n, int& i0, float& f) {
     if (CLAMP) u = fminf(fmaxf(u, 0.5f), static_cast<float>(n) + 0.5f);
-    const float fl = floorf(u);
-    i0 = static_cast<int>(fl);
-    f = u - fl;
+    i0 = __float2int_rd(u);
+    f = u - floorf(u);
 }
 
 // x-lerp of two FP16 corners read raw (four halves each), in FP32: the first
@@ -410,29 +418,59 @@ __device__ __forceinline__ float3 renormalize(float3 w1, float3 d1) {
     return fma3(renorm_term(w1), w1, d1);
 }
 
+// Two neighbouring RGB8 texels, six bytes from p on, from the aligned 32-bit
+// words that hold them (no word without a byte of them is read): two loads, or
+// three where p is the last byte of a word, instead of six.
+__device__ __forceinline__ void texel_pair(const uint8_t* __restrict__ p, float2& r, float2& g,
+                                           float2& b) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    const unsigned* w = reinterpret_cast<const unsigned*>(at & ~uintptr_t(3));
+    const unsigned byte = static_cast<unsigned>(at) & 3u;
+    const unsigned w0 = __ldg(w), w1 = __ldg(w + 1), w2 = byte == 3u ? __ldg(w + 2) : 0u;
+    const unsigned lo = __funnelshift_r(w0, w1, 8u * byte), hi = __funnelshift_r(w1, w2, 8u * byte);
+    r = make_float2(static_cast<float>(lo & 0xFFu), static_cast<float>(lo >> 24));
+    g = make_float2(static_cast<float>((lo >> 8) & 0xFFu), static_cast<float>(hi & 0xFFu));
+    b = make_float2(static_cast<float>((lo >> 16) & 0xFFu), static_cast<float>((hi >> 8) & 0xFFu));
+}
+
+// Bilinear colour of texel pairs p0 (row j) and p1 (row j + 1); value / 255.
+__device__ __forceinline__ float3 texel_lerp(const uint8_t* __restrict__ p0,
+                                             const uint8_t* __restrict__ p1, float fs, float ft) {
+    float2 r0, g0, b0, r1, g1, b1;
+    texel_pair(p0, r0, g0, b0);
+    texel_pair(p1, r1, g1, b1);
+    constexpr float k = 1.0f / 255.0f;
+    return make_float3(lerpf(lerpf(r0.x, r0.y, fs), lerpf(r1.x, r1.y, fs), ft) * k,
+                       lerpf(lerpf(g0.x, g0.y, fs), lerpf(g1.x, g1.y, fs), ft) * k,
+                       lerpf(lerpf(b0.x, b0.y, fs), lerpf(b1.x, b1.y, fs), ft) * k);
+}
+
 // Colour of direction d in the equirect environment map (bilinear, u wraps,
 // v clamps; value / 255).
 __device__ __forceinline__ float3 environment(const VolArgs& A, float3 d) {
     const float phi = atan2f(d.y, d.x);
     const float theta = atan2f(sqrtf(fmaf(d.y, d.y, d.x * d.x)), d.z);
     const float W = static_cast<float>(A.bgW), H = static_cast<float>(A.bgH);
-    const float u = fmaf(phi, W / (2.0f * kPi), 0.5f * W - 0.5f);
-    float v = fmaf(theta, H / kPi, -0.5f);
+    const float u = fmaf(phi, A.bg_u, 0.5f * W - 0.5f);
+    float v = fmaf(theta, A.bg_v, -0.5f);
     const float ufl = floorf(u);
     const float fu = u - ufl;
-    int i0 = static_cast<int>(ufl) % A.bgW;
+    // |phi| is at most pi (to a rounding): u lies within a texel of [0, W)
+    int i0 = static_cast<int>(ufl);
     if (i0 < 0) i0 += A.bgW;
-    const int i1 = (i0 + 1 == A.bgW) ? 0 : i0 + 1;
+    if (i0 >= A.bgW) i0 -= A.bgW;
     v = fminf(fmaxf(v, 0.0f), H - 1.0f);
     const int j0 = min(static_cast<int>(floorf(v)), A.bgH - 2);
     const float fv = v - static_cast<float>(j0);
     const uint8_t* r0 = A.bg + static_cast<size_t>(j0) * A.bgW * 3;
     const uint8_t* r1 = r0 + static_cast<size_t>(A.bgW) * 3;
+    if (i0 + 1 < A.bgW) return texel_lerp(r0 + 3 * i0, r1 + 3 * i0, fu, fv);
+    // the pair that wraps: the last texel of a row and its first
     float out[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float t00 = __ldg(r0 + i0 * 3 + c), t01 = __ldg(r0 + i1 * 3 + c);
-        const float t10 = __ldg(r1 + i0 * 3 + c), t11 = __ldg(r1 + i1 * 3 + c);
+        const float t00 = __ldg(r0 + i0 * 3 + c), t01 = __ldg(r0 + c);
+        const float t10 = __ldg(r1 + i0 * 3 + c), t11 = __ldg(r1 + c);
         out[c] = lerpf(lerpf(t00, t01, fu), lerpf(t10, t11, fu), fv) * (1.0f / 255.0f);
     }
     return make_float3(out[0], out[1], out[2]);
@@ -450,15 +488,7 @@ __device__ __forceinline__ float3 texel_bilinear(const uint8_t* tex, int W, int 
     const int j0 = min(static_cast<int>(floorf(t)), H - 2);
     const float fs = s - static_cast<float>(i0), ft = t - static_cast<float>(j0);
     const uint8_t* r0 = tex + (static_cast<size_t>(j0) * W + i0) * 3;
-    const uint8_t* r1 = r0 + static_cast<size_t>(W) * 3;
-    float out[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const float t00 = __ldg(r0 + c), t01 = __ldg(r0 + 3 + c);
-        const float t10 = __ldg(r1 + c), t11 = __ldg(r1 + 3 + c);
-        out[c] = lerpf(lerpf(t00, t01, fs), lerpf(t10, t11, fs), ft) * (1.0f / 255.0f);
-    }
-    return make_float3(out[0], out[1], out[2]);
+    return texel_lerp(r0, r0 + static_cast<size_t>(W) * 3, fs, ft);
 }
 
 // What the straight ray P + t d (t > 0) sees: the nearest textured plane it
@@ -795,7 +825,7 @@ __device__ __forceinline__ void ray_end(const VolArgs& V, const ViewArgs& C, int
 // One view, one thread per pixel: a block of 128 threads covers 16x8 pixels,
 // each warp an 8x4 tile.
 template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
-__global__ void __launch_bounds__(128, (STEPPER == HH_STEP_RK4) ? 6 : HH_MARCH_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, march_blocks(STEPPER))
     march_kernel(const VolArgs V, const ViewArgs C) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int tx, ty;
@@ -811,16 +841,19 @@ __global__ void __launch_bounds__(128, (STEPPER == HH_STEP_RK4) ? 6 : HH_MARCH_M
     ray_end(V, C, px, py, R, ep, ed);
 }
 
-// View and view-local index of batch tile t: from the order table when
-// there is one (tiles of all views in the order the table gives), else the
-// last view whose first tile is <= t (views one after the other).
+// View and place (column, row of tiles) of batch tile t: from the order table
+// when there is one ({view, row << 16 | column}, the tiles of all views in the
+// order the table gives; a view has at most 2^15 rows and 2^14 columns), else
+// in the last view whose first tile is <= t (views one after the other).
 __device__ __forceinline__ void tile_of(int t, int n_views, const int* s_begin,
-                                        const uint2* __restrict__ order, int& view,
-                                        int& local) {
+                                        const ViewArgs* __restrict__ views,
+                                        const uint2* __restrict__ order, int& view, int& tx,
+                                        int& ty) {
     if (order) {
         const uint2 o = __ldg(order + t);
         view = static_cast<int>(o.x);
-        local = static_cast<int>(o.y);
+        tx = static_cast<int>(o.y & 0xFFFFu);
+        ty = static_cast<int>(o.y >> 16);
         return;
     }
     int lo = 0, hi = n_views - 1;
@@ -830,7 +863,9 @@ __device__ __forceinline__ void tile_of(int t, int n_views, const int* s_begin,
         else hi = mid - 1;
     }
     view = lo;
-    local = t - s_begin[lo];
+    const int local = t - s_begin[lo], tiles_x = __ldg(&views[lo].tiles_x);
+    ty = local / tiles_x;
+    tx = local - ty * tiles_x;
 }
 
 // Persistent batched march over many views of uneven size. Each warp pulls
@@ -848,7 +883,7 @@ __device__ __forceinline__ void tile_of(int t, int n_views, const int* s_begin,
 // before the next group, as march_kernel's blocks do when they retire. The
 // per-ray arithmetic is march_kernel's.
 template <int STORAGE, int STEPPER, bool ADAPTIVE, bool REFILL, int ADDR>
-__global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_MIN_BLOCKS)
+__global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
     march_batch_kernel(const VolArgs V, const ViewArgs* __restrict__ views, int n_views,
                        int total_tiles, int tile_w, unsigned* __restrict__ counter,
                        int refill_min, const uint2* __restrict__ order, int group) {
@@ -863,7 +898,13 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
     const unsigned sparse = __ldg(V.sparse);
     if (!REFILL) {
         __shared__ int s_group;  // first tile of the block's current group
+        // the warps' current view records: one coalesced load where the view
+        // changes, instead of a load per field and tile
+        __shared__ ViewArgs s_view[8];
+        constexpr int kWords = sizeof(ViewArgs) / sizeof(unsigned);
         const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+        ViewArgs& C = s_view[warp];
+        int have_view = -1;
         int lx, ly;
         tile_pixel(lane, tile_w_log2, lx, ly);
         for (;;) {
@@ -881,10 +922,16 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
                 t = __shfl_sync(FULL, t, 0);
                 if (t >= total_tiles) return;
             }
-            int lo, local;
-            tile_of(t, n_views, s_begin, order, lo, local);
-            const ViewArgs& C = views[lo];
-            const int ty = local / C.tiles_x, tx = local - ty * C.tiles_x;
+            int view, tx, ty;
+            tile_of(t, n_views, s_begin, views, order, view, tx, ty);
+            if (view != have_view) {  // warp-uniform
+                __syncwarp();         // the last tile's reads are done
+                const unsigned* src = reinterpret_cast<const unsigned*>(views + view);
+                for (int w = lane; w < kWords; w += 32)
+                    reinterpret_cast<unsigned*>(&C)[w] = __ldg(src + w);
+                __syncwarp();
+                have_view = view;
+            }
             const int px = (tx << tile_w_log2) + lx, py = ty * (32 >> tile_w_log2) + ly;
             if (px < C.W && py < C.H) {
                 RayState R;
@@ -896,7 +943,7 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
             }
         }
     }
-    int tile_local = 0, tile_view = 0, pos = 32;  // the warp's pixel stream (warp-uniform)
+    int tile_x = 0, tile_y = 0, tile_view = 0, pos = 32;  // the warp's pixel stream (warp-uniform)
     bool done = false, have = false;
     int vi = 0, px = 0, py = 0;
     RayState R;
@@ -914,7 +961,7 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
                         done = true;
                         break;
                     }
-                    tile_of(t, n_views, s_begin, order, tile_view, tile_local);
+                    tile_of(t, n_views, s_begin, views, order, tile_view, tile_x, tile_y);
                     pos = 0;
                 }
                 const int avail = 32 - pos;
@@ -922,13 +969,11 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_BATCH_M
                 const bool mine = ((todo >> lane) & 1u) && rank < avail;
                 if (mine) {
                     const ViewArgs& C = views[tile_view];
-                    const int local = tile_local;
                     const int p = pos + rank;
-                    const int ty = local / C.tiles_x, tx = local - ty * C.tiles_x;
                     int lx, ly;
                     tile_pixel(p, tile_w_log2, lx, ly);
-                    px = (tx << tile_w_log2) + lx;
-                    py = ty * (32 >> tile_w_log2) + ly;
+                    px = (tile_x << tile_w_log2) + lx;
+                    py = tile_y * (32 >> tile_w_log2) + ly;
                     vi = tile_view;
                     if (px < C.W && py < C.H) {
                         ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
@@ -992,20 +1037,33 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// Resident 256-thread blocks per SM of the serving worker: 4 (64 registers)
-// for the Eq. 16 march, whose per-tile and per-job state lives outside the
-// step loop.
-#ifndef HH_WORKER_MIN_BLOCKS
-#define HH_WORKER_MIN_BLOCKS 4
-#endif
+// What a warp of the serving worker keeps between tiles, in shared memory: the
+// view record of its current tile and its job. In registers the march's loop
+// spilled (six requests of three views on a 384^3 FP16 volume: 12.2 against 11.4
+// ms).
+struct alignas(16) WorkerWarp {
+    ViewArgs view;
+    unsigned long long vol, scales;  // addresses of the job's volume and its FP16 scales
+    unsigned sparse;
+    int view_begin, n_views, n_tiles;
+    int view_first, view_end;  // job-relative tiles of the view held
+};
+
+// Resident 256-thread blocks per SM of the serving worker: as the batched
+// kernel's (FP16: 5 against 4, six requests of three views on a 384^3 volume in
+// 10.65 against 11.4 ms).
+constexpr int worker_blocks(int storage, int stepper) {
+    return batch_blocks(storage, stepper, false);
+}
 
 template <int STORAGE, int STEPPER, bool ADAPTIVE>
-__global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_MIN_BLOCKS)
+__global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
     serve_worker_kernel(const VolArgs V, const ServeWorkerArgs W) {
-    extern __shared__ __align__(16) unsigned char s_raw[];  // one view record per warp
+    extern __shared__ __align__(16) unsigned char s_raw[];  // a WorkerWarp per warp
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ViewArgs& C = reinterpret_cast<ViewArgs*>(s_raw)[warp];
+    WorkerWarp& S = reinterpret_cast<WorkerWarp*>(s_raw)[warp];
+    ViewArgs& C = S.view;
     const int tile_w_log2 = W.tile_w == 16 ? 4 : (W.tile_w == 8 ? 3 : 2);
     const int tile_h = 32 >> tile_w_log2;
     int lx, ly;
@@ -1014,11 +1072,6 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
     constexpr int kWords = sizeof(ViewArgs) / sizeof(unsigned);
     int j = ld_acquire_int(W.first_open);
     int have_job = -1;
-    int view_first = 0, view_end = 0;  // job-relative tiles of the view in C
-    const void* jvol = nullptr;
-    const float* jscales = nullptr;
-    unsigned jsparse = 0;
-    int jview_begin = 0, jn_views = 0, jn_tiles = 0;
     unsigned t = 0;  // this warp's claimed tile of job j (valid while have_job == j)
     bool claimed_next = false;
     unsigned long long idle_since = 0;
@@ -1089,18 +1142,20 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
                 if (lane == 0) atomicSub(W.idle_warps, 1);
                 counted_idle = false;
             }
-            const ServeJob* e = W.jobs + j;
-            jvol = reinterpret_cast<const void*>(
-                __ldcg(reinterpret_cast<const unsigned long long*>(&e->vol)));
-            jscales = reinterpret_cast<const float*>(
-                __ldcg(reinterpret_cast<const unsigned long long*>(&e->scales)));
-            jsparse = __ldcg(reinterpret_cast<const unsigned*>(
-                __ldcg(reinterpret_cast<const unsigned long long*>(&e->sparse))));
-            jview_begin = __ldcg(&e->view_begin);
-            jn_views = __ldcg(&e->n_views);
-            jn_tiles = __ldcg(&e->n_tiles);
+            __syncwarp();
+            if (lane == 0) {
+                const ServeJob* e = W.jobs + j;
+                S.vol = __ldcg(reinterpret_cast<const unsigned long long*>(&e->vol));
+                S.scales = __ldcg(reinterpret_cast<const unsigned long long*>(&e->scales));
+                S.sparse = __ldcg(reinterpret_cast<const unsigned*>(
+                    __ldcg(reinterpret_cast<const unsigned long long*>(&e->sparse))));
+                S.view_begin = __ldcg(&e->view_begin);
+                S.n_views = __ldcg(&e->n_views);
+                S.n_tiles = __ldcg(&e->n_tiles);
+                S.view_first = S.view_end = 0;
+            }
+            __syncwarp();
             have_job = j;
-            view_first = view_end = 0;
             claimed_next = false;
         }
         if (!claimed_next) {
@@ -1108,39 +1163,43 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
             t = __shfl_sync(FULL, t, 0);
         }
         claimed_next = false;
-        if (t >= static_cast<unsigned>(jn_tiles)) {  // exhausted (or failed): next job
+        if (t >= static_cast<unsigned>(S.n_tiles)) {  // exhausted (or failed): next job
             ++j;
             if (lane == 0) atomicMax(W.first_open, j);
             continue;
         }
         const int ti = static_cast<int>(t);
-        if (ti < view_first || ti >= view_end) {
+        if (ti < S.view_first || ti >= S.view_end) {
             // the tile's view: the last view of the job whose first tile is <= t
-            int lo = 0, hi = jn_views - 1;
+            int lo = 0, hi = S.n_views - 1;
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
                 const ViewArgs* vm = reinterpret_cast<const ViewArgs*>(
-                    views + static_cast<size_t>(jview_begin + mid) * sizeof(ViewArgs));
+                    views + static_cast<size_t>(S.view_begin + mid) * sizeof(ViewArgs));
                 if (__ldcg(&vm->tile_begin) <= ti) lo = mid;
                 else hi = mid - 1;
             }
             __syncwarp();
             const unsigned* src = reinterpret_cast<const unsigned*>(
-                views + static_cast<size_t>(jview_begin + lo) * sizeof(ViewArgs));
+                views + static_cast<size_t>(S.view_begin + lo) * sizeof(ViewArgs));
             for (int w = lane; w < kWords; w += 32) reinterpret_cast<unsigned*>(&C)[w] = __ldcg(src + w);
             __syncwarp();
-            view_first = C.tile_begin;
-            view_end = view_first + C.tiles_x * ((C.H + tile_h - 1) / tile_h);
+            if (lane == 0) {
+                S.view_first = C.tile_begin;
+                S.view_end = C.tile_begin + C.tiles_x * ((C.H + tile_h - 1) / tile_h);
+            }
+            __syncwarp();
         }
-        const int local = ti - view_first;
+        const int local = ti - S.view_first;
         const int ty = local / C.tiles_x, tx = local - ty * C.tiles_x;
         const int px = (tx << tile_w_log2) + lx, py = ty * tile_h + ly;
         if (px < C.W && py < C.H) {
             RayState R;
             float3 ep = make_float3(0.0f, 0.0f, 0.0f), ed = ep;
-            ray_begin<ADAPTIVE>(V, jscales, C, px, py, R);
+            ray_begin<ADAPTIVE>(V, reinterpret_cast<const float*>(S.scales), C, px, py, R);
             if (R.flags & HH_FLAG_HIT)
-                ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>(V, jvol, jsparse, R, ep, ed);
+                ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>(
+                    V, reinterpret_cast<const void*>(S.vol), S.sparse, R, ep, ed);
             ray_end(V, C, px, py, R, ep, ed);
         }
         // count the tile (release: its outputs are ordered before the count,
@@ -1154,7 +1213,7 @@ __global__ void __launch_bounds__(256, (STEPPER == HH_STEP_RK4) ? 3 : HH_WORKER_
             const unsigned before = atom_add_acq_rel(W.done + j, 1u);
             leave = ld_acquire_int(W.leave);
             if (!leave) next = atomicAdd(W.claimed + j, 1u);
-            if (before + 1u == static_cast<unsigned>(jn_tiles)) {
+            if (before + 1u == static_cast<unsigned>(S.n_tiles)) {
                 __threadfence_system();
                 W.host_done[j] = HH_JOB_DONE;
             }
@@ -1227,7 +1286,7 @@ template <int ST, int SP, bool AD>
 struct WorkerLaunch {
     static void run(const VolArgs& V, const ServeWorkerArgs& W, int blocks, int threads,
                     cudaStream_t s) {
-        const size_t smem = (threads / 32) * sizeof(ViewArgs);
+        const size_t smem = (threads / 32) * sizeof(WorkerWarp);
         serve_worker_kernel<ST, SP, AD><<<blocks, threads, smem, s>>>(V, W);
     }
 };
@@ -1236,7 +1295,7 @@ template <int ST, int SP, bool AD>
 struct WorkerOccupancy {
     static void run(int threads, int* blocks_per_sm) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, serve_worker_kernel<ST, SP, AD>,
-                                                      threads, (threads / 32) * sizeof(ViewArgs));
+                                                      threads, (threads / 32) * sizeof(WorkerWarp));
     }
 };
 
@@ -1284,6 +1343,8 @@ VolArgs make_vol_args(const hh_volume_s* vol, const hh_step_params& P, const hh_
     A.bg = bg.rgb8_dev;
     A.bgW = bg.width;
     A.bgH = bg.height;
+    A.bg_u = static_cast<float>(bg.width) / (2.0f * kPi);
+    A.bg_v = static_cast<float>(bg.height) / kPi;
     A.n_planes = bg.n_planes;
     for (int k = 0; k < HH_MAX_PLANES; ++k) A.planes[k] = bg.planes[k];
     return A;
@@ -1416,7 +1477,7 @@ void drop_graph(hh_batch b) {
 std::vector<uint2> interleaved_order(const std::vector<hh::ViewArgs>& v, int tile_w) {
     struct Key {
         double k;
-        uint32_t view, local;
+        uint32_t view, place;  // place: row << 16 | column
     };
     std::vector<Key> keys;
     const int tile_h = 32 / tile_w;
@@ -1425,11 +1486,11 @@ std::vector<uint2> interleaved_order(const std::vector<hh::ViewArgs>& v, int til
         for (int ty = 0; ty < tiles_y; ++ty)
             for (int tx = 0; tx < v[i].tiles_x; ++tx)
                 keys.push_back({(ty + 0.5) / tiles_y, static_cast<uint32_t>(i),
-                                static_cast<uint32_t>(ty * v[i].tiles_x + tx)});
+                                static_cast<uint32_t>(ty) << 16 | static_cast<uint32_t>(tx)});
     }
     std::stable_sort(keys.begin(), keys.end(), [](const Key& x, const Key& y) { return x.k < y.k; });
     std::vector<uint2> ord(keys.size());
-    for (size_t j = 0; j < keys.size(); ++j) ord[j] = make_uint2(keys[j].view, keys[j].local);
+    for (size_t j = 0; j < keys.size(); ++j) ord[j] = make_uint2(keys[j].view, keys[j].place);
     return ord;
 }
 
