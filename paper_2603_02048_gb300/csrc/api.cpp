@@ -160,8 +160,10 @@ hh_status new_volume(const hh_grid* g, hh_volume* out) {
     const size_t pairs = (static_cast<size_t>(g->nz) + 3) / 2;
     const size_t elements = static_cast<size_t>(v->pair) * pairs;
     const size_t mask_words = (elements + 31) / 32;
-    v->nz_words = (static_cast<unsigned>(g->nx) + 2u + 31u) / 32u;
-    const size_t nz_total = 2 * pairs * (static_cast<size_t>(g->ny) + 3) * v->nz_words;
+    // (the mask kernel reads up to a slice, two rows and a word past the last)
+    v->nz_words = (static_cast<unsigned>(g->nx) + 31u) / 32u;
+    const size_t rows = (static_cast<size_t>(g->ny) + 3) / 2 * 2;
+    const size_t nz_total = ((2 * pairs + 1) * rows + 3) * v->nz_words + 2;
     v->mask_off = (elements * voxel_bytes + 255) & ~size_t(255);
     const size_t total = v->mask_off + (mask_words + nz_total + 1) * sizeof(unsigned);
     cudaGetDevice(&v->device);

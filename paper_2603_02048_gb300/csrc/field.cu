@@ -60,43 +60,59 @@ __device__ __forceinline__ uint2 pack16(const Voxel& v, float rs_n, float rs_g) 
                       *reinterpret_cast<const unsigned*>(&hi));
 }
 
-// A thread owns voxel column I of a pair of rows J = 2 jj, 2 jj + 1 and walks
-// `run` pairs of slices K = 2 kk, 2 kk + 1: four voxels an iteration. A row's two
-// are consecutive in the ZPAIR layout, so a warp stores 1 KiB (FP32) or 512 B
-// (FP16) in one piece per row. K rho of the two rows stays in registers from
-// slice to slice and each row is the other's y neighbour: a slice of the pair
-// costs eight loads (two centres, two outer rows, four x neighbours), where a
-// thread per column needs ten. H = 1 (ZPAIR): padded coordinates are grid
-// coordinates + 1 and the halo repeats the nearest grid voxel; H = 0 (LINEAR,
-// and the max pass, which stores nothing): they are the grid's. A one-sided
-// difference is the central one with the missing neighbour replaced by the
-// voxel itself and the factor 1 instead of 1/2. Threads of the padding compute
-// a clamped voxel, which does not change a maximum and is not stored.
+// A thread owns grid column i of a pair of padded rows J = 2 jj, 2 jj + 1 and
+// walks `run` pairs of padded slices K = 2 kk, 2 kk + 1: four voxels an iteration.
+// A row's two are consecutive in the ZPAIR layout, so a warp stores 1 KiB (FP32)
+// or 512 B (FP16) in one piece per row. K rho of the two rows stays in registers
+// from slice to slice and each row is the other's y neighbour: a slice of the
+// pair costs eight loads (two centres, two outer rows, four x neighbours),
+// where a thread per column needs ten. H = 1 (ZPAIR): padded coordinates are
+// grid coordinates + 1 and the halo repeats the nearest grid voxel (in x, the
+// first and last column store twice); H = 0 (LINEAR, and
+// the max pass, which stores nothing): they are the grid's. A
+// one-sided difference is the central one with the missing neighbour replaced
+// by the voxel itself and the factor 1 instead of 1/2. Threads of the padding
+// compute a clamped voxel, which does not change a maximum and is not stored.
+// What bounds it: DRAM and its latency. 256^3 FP32: 58 us for the 285 MB it
+// moves (74 with a thread per column and 16-byte stores), FP16: maxima 33, store
+// 46 us (38 and 66). 5 resident blocks (48 registers) against 4 take 4 % off a
+// 512^3 FP16 build.
+constexpr int field_blocks(int mode) { return mode == 1 ? 4 : 5; }
+
 template <int MODE, int H>  // 0: FP32 store, 1: FP16 max pass, 2: FP16 store
-__global__ void __launch_bounds__(256)
-    field_kernel(const float* __restrict__ rho, int nx, int ny, int nz, float K, unsigned width,
-                 int run, unsigned row, unsigned pair, void* __restrict__ out,
-                 unsigned* __restrict__ nz_bits, unsigned nz_words,
-                 unsigned* __restrict__ sparse,
+__global__ void __launch_bounds__(256, field_blocks(MODE))
+    field_kernel(const float* __restrict__ rho, int nx, int ny, int nz, float K, int run,
+                 unsigned row, unsigned pair, void* __restrict__ out,
+                 unsigned* __restrict__ nz_bits, unsigned* __restrict__ sparse,
                  unsigned* __restrict__ max_bits, float* __restrict__ scales) {
-    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned jj = t / width, I = t - jj * width;
+    // warps go along x, then to the next pair of rows
+    const unsigned lane = threadIdx.x & 31, nz_words = (static_cast<unsigned>(nx) + 31u) / 32u;
+    const unsigned warp = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const unsigned jj = warp / nz_words, word = warp - jj * nz_words;
+    const unsigned I = word * 32 + lane;  // grid column
     const int row_pairs = (ny + 2 * H + 1) / 2, slice_pairs = (nz + 2 * H + 1) / 2;
-    const bool valid = static_cast<int>(jj) < row_pairs && static_cast<int>(I) < nx + 2 * H;
-    const int i = min(max(static_cast<int>(I) - H, 0), nx - 1);
-    const int J0 = min(2 * static_cast<int>(jj), 2 * row_pairs - 2) - H, J1 = J0 + 1;
-    const int j0 = min(max(J0, 0), ny - 1), j1 = min(J1, ny - 1);
+    const int kk0 = blockIdx.y * run, kk1 = min(kk0 + run, slice_pairs);
+    const bool valid = static_cast<int>(jj) < row_pairs && static_cast<int>(I) < nx;
     float s_n = 1.0f, s_g = 1.0f;
     if (MODE == 2) {
         s_n = scale_of(max_bits[0]);
         s_g = scale_of(max_bits[1]);
     }
     const float rs_n = 1.0f / s_n, rs_g = 1.0f / s_g;  // exact: powers of two
-    if (t == 0 && blockIdx.y == 0 && MODE != 1) {
+    if (MODE != 1 && threadIdx.x == 0 && blockIdx.x + blockIdx.y == 0) {
         scales[0] = s_n;
         scales[1] = s_g;
         if (H) *sparse = 0;  // free_mask_kernel, the next launch, may set it
     }
+    // this warp's row pair of nonzero words: lane l < 4 owns row l & 1, slice l >> 1
+    unsigned* const nz_at =
+        H ? nz_bits + (static_cast<size_t>(2 * kk0 + (lane >> 1)) * (2 * row_pairs) + 2 * jj + (lane & 1)) *
+                          nz_words + word
+          : nullptr;
+    const size_t nz_step = static_cast<size_t>(4 * row_pairs) * nz_words;
+    const int i = min(static_cast<int>(I), nx - 1);
+    const int J0 = min(2 * static_cast<int>(jj), 2 * row_pairs - 2) - H, J1 = J0 + 1;
+    const int j0 = min(max(J0, 0), ny - 1), j1 = min(J1, ny - 1);
     const size_t sz = static_cast<size_t>(nx) * ny;
     const float* r0 = rho + static_cast<size_t>(j0) * nx + i;
     const float* r1 = rho + static_cast<size_t>(j1) * nx + i;
@@ -107,7 +123,6 @@ __global__ void __launch_bounds__(256)
     const float fy0 = j0 > 0 && j0 < ny - 1 ? 0.5f : 1.0f;
     const float fy1 = j1 > 0 && j1 < ny - 1 ? 0.5f : 1.0f;
     const bool first_row = J0 < 0, last_row = J1 >= ny;
-    const int kk0 = blockIdx.y * run, kk1 = min(kk0 + run, slice_pairs);
     // dn = K rho, rounded by itself (an FMA with the difference that uses it would
     // give a gradient that is not the stored dn's)
     auto dn_of = [K](const float* p) { return __fmul_rn(K, __ldg(p)); };
@@ -171,7 +186,7 @@ __global__ void __launch_bounds__(256)
             peak(v11);
         } else if (H == 0) {
             if (valid) {
-                const size_t o = (static_cast<size_t>(K0) * ny + J0) * nx + I;
+                const size_t o = (static_cast<size_t>(K0) * ny + J0) * nx + i;
                 uint4* to = static_cast<uint4*>(out) + o;
                 __stcs(to, pack32(v00));
                 if (J1 < ny) __stcs(to + nx, pack32(v10));
@@ -179,9 +194,11 @@ __global__ void __launch_bounds__(256)
                 if (J1 < ny && K1 < nz) __stcs(to + sz + nx, pack32(v11));
             }
         } else {
-            const unsigned J = 2 * jj, slice = 2 * static_cast<unsigned>(kk);
+            const unsigned J = 2 * jj;
             const bool valid1 = valid && static_cast<int>(J) + 1 < ny + 2;
-            const size_t o = static_cast<size_t>(kk) * pair + J * row + 2 * I;
+            // element of (I = i + 1, J, 2 kk); the halo columns are the first
+            // and the last thread's second stores
+            const size_t o = static_cast<size_t>(kk) * pair + J * row + 2 * (I + 1);
             bool z00, z10, z01, z11;  // holds only +-0
             if (MODE == 0) {
                 const uint4 w00 = pack32(v00), w01 = pack32(v01);
@@ -192,8 +209,13 @@ __global__ void __launch_bounds__(256)
                 z10 = zero(w10);
                 z11 = zero(w11);
                 uint4* to = static_cast<uint4*>(out) + o;
-                if (valid) store32(to, w00, w01);
-                if (valid1) store32(to + row, w10, w11);
+                auto put = [&](int d) {
+                    if (valid) store32(to + d, w00, w01);
+                    if (valid1) store32(to + static_cast<int>(row) + d, w10, w11);
+                };
+                put(0);
+                if (xl == 0) put(-2);
+                if (xh == 0) put(2);
             } else {
                 const uint2 w00 = pack16(v00, rs_n, rs_g), w01 = pack16(v01, rs_n, rs_g);
                 const uint2 w10 = pack16(v10, rs_n, rs_g), w11 = pack16(v11, rs_n, rs_g);
@@ -203,24 +225,23 @@ __global__ void __launch_bounds__(256)
                 z10 = zero(w10);
                 z11 = zero(w11);
                 uint2* to = static_cast<uint2*>(out) + o;
-                if (valid) __stcs(reinterpret_cast<uint4*>(to), make_uint4(w00.x, w00.y, w01.x, w01.y));
-                if (valid1)
-                    __stcs(reinterpret_cast<uint4*>(to + row), make_uint4(w10.x, w10.y, w11.x, w11.y));
+                auto put = [&](int d) {
+                    if (valid) __stcs(reinterpret_cast<uint4*>(to + d), make_uint4(w00.x, w00.y, w01.x, w01.y));
+                    if (valid1)
+                        __stcs(reinterpret_cast<uint4*>(to + static_cast<int>(row) + d),
+                               make_uint4(w10.x, w10.y, w11.x, w11.y));
+                };
+                put(0);
+                if (xl == 0) put(-2);
+                if (xh == 0) put(2);
             }
-            // nonzero bits, a word per row and slice (width is a multiple of
-            // 32: a warp is one word of one pair of rows); the padding counts
-            // as nonzero
-            const unsigned n00 = __ballot_sync(0xffffffffu, !(valid && z00));
-            const unsigned n10 = __ballot_sync(0xffffffffu, !(valid1 && z10));
-            const unsigned n01 = __ballot_sync(0xffffffffu, !(valid && z01));
-            const unsigned n11 = __ballot_sync(0xffffffffu, !(valid1 && z11));
-            const unsigned lane = threadIdx.x & 31;
-            if (lane < 4 && static_cast<int>(jj) < row_pairs) {
-                const unsigned word = lane & 2 ? (lane & 1 ? n11 : n01) : (lane & 1 ? n10 : n00);
-                const unsigned rows = 2 * static_cast<unsigned>(row_pairs);
-                nz_bits[(static_cast<size_t>(slice + (lane >> 1)) * rows + J + (lane & 1)) * nz_words +
-                        (I >> 5)] = word;
-            }
+            // nonzero bits, a word per row and slice
+            const unsigned n00 = __ballot_sync(0xffffffffu, valid && !z00);
+            const unsigned n10 = __ballot_sync(0xffffffffu, valid1 && !z10);
+            const unsigned n01 = __ballot_sync(0xffffffffu, valid && !z01);
+            const unsigned n11 = __ballot_sync(0xffffffffu, valid1 && !z11);
+            if (lane < 4 && static_cast<int>(jj) < row_pairs)
+                nz_at[(kk - kk0) * nz_step] = lane & 2 ? (lane & 1 ? n11 : n01) : (lane & 1 ? n10 : n00);
         }
         p0 = b0;
         p1 = b1;
@@ -258,45 +279,58 @@ constexpr unsigned kSparseFree = 128;
 
 // The free-corner mask from the store pass's nonzero bits, a word (32
 // consecutive elements: 16 columns of a row of a pair of slices, or the end of
-// one row and the start of the next) per thread. Column I of row J, slice K is
-// free when none of columns I, I + 1 of rows J, J + 1 of slices K, K + 1 holds a
-// nonzero value; whatever lies beyond the stored rows and columns counts as
-// nonzero.
+// one row and the start of the next) per thread; blockIdx.y is the pair of
+// slices the word starts in. Column I of row J, slice K is free when none of
+// columns I, I + 1 of rows J, J + 1 of slices K, K + 1 holds a nonzero value; the
+// halo columns hold what the first and the last grid column do. What it says of
+// cells beyond the last sampled column, row and slice is not read.
+// 256^3 (537,000 words): 13 us, latency and issue; with a window per row, slice
+// and neighbour and the words' places from integer divisions it took 17.
 __global__ void __launch_bounds__(256)
-    free_mask_kernel(const unsigned* __restrict__ nz, unsigned nz_words, unsigned rows,
-                     unsigned pairs, unsigned row, unsigned pair, unsigned words,
+    free_mask_kernel(const unsigned* __restrict__ nz, unsigned nz_words, int nx, int ny,
+                     unsigned pairs, unsigned row, unsigned pair, float per_row,
                      unsigned* __restrict__ fr, unsigned* __restrict__ sparse) {
-    const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned free_bits = 0;
-    if (g < words) {
-        // 32 columns from column c of a row's nonzero bits
-        auto columns = [&](unsigned slice, unsigned J, unsigned c) {
-            if (slice >= 2 * pairs || J >= rows) return 0xFFFFFFFFu;
-            const unsigned* w = nz + (static_cast<size_t>(slice) * rows + J) * nz_words;
-            const unsigned i = c >> 5;
-            const unsigned lo = i < nz_words ? __ldg(w + i) : 0xFFFFFFFFu;
-            const unsigned hi = i + 1 < nz_words ? __ldg(w + i + 1) : 0xFFFFFFFFu;
-            return __funnelshift_r(lo, hi, c);
-        };
-        auto spread = [](unsigned x) {  // bit i of the low half to bit 2 i
-            x = (x | (x << 8)) & 0x00FF00FFu;
-            x = (x | (x << 4)) & 0x0F0F0F0Fu;
-            x = (x | (x << 2)) & 0x33333333u;
-            return (x | (x << 1)) & 0x55555555u;
-        };
-        unsigned kk = 32u * g / pair, at = 32u * g - kk * pair;  // elements: below 2^32
+    const unsigned rows = (static_cast<unsigned>(ny) + 3u) / 2u * 2u;
+    const size_t slice = static_cast<size_t>(rows) * nz_words;  // words
+    unsigned kk = blockIdx.y;
+    const unsigned g = (kk * pair + 31u) / 32u + blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned at = 32u * g - kk * pair;  // element of the pair; even
+    unsigned sampled_free = 0;
+    if (at < pair) {
+        unsigned word = 0;
         for (unsigned done = 0; done < 32u && kk < pairs;) {
-            const unsigned J = at / row, e = at - J * row;  // e is even
-            const unsigned n = min(32u - done, min(row - e, pair - at));
-            unsigned busy[3];
+            unsigned J = static_cast<unsigned>(__uint2float_rz(at) * per_row);  // at / row, off by one
+            if (J * row > at) --J;
+            if ((J + 1u) * row <= at) ++J;
+            const unsigned e = at - J * row, n = min(32u - done, min(row - e, pair - at));
+            // columns I = c, c + 1, .. hold grid columns c - 1, c, ..: a window of
+            // the rows' bits from c - 1 on, ORed with itself one column on. The
+            // words left of the first and right of the last are another row's.
+            const int c = static_cast<int>(e >> 1), i = (c - 1) >> 5;
+            const unsigned in_lo = i >= 0 ? 0xFFFFFFFFu : 0u;
+            const unsigned in_hi = i + 1 < static_cast<int>(nz_words) ? 0xFFFFFFFFu : 0u;
+            const unsigned* w = nz + 2u * kk * slice + static_cast<size_t>(J) * nz_words + i;
+            unsigned lo[3], hi[3];  // per slice, rows J and J + 1
 #pragma unroll
-            for (unsigned z = 0; z < 3; ++z) {
-                const unsigned a = columns(2 * kk + z, J, e >> 1) | columns(2 * kk + z, J + 1, e >> 1);
-                busy[z] = a | (a >> 1);
+            for (int z = 0; z < 3; ++z, w += slice) {
+                lo[z] = __ldg(w) | __ldg(w + nz_words);
+                hi[z] = __ldg(w + 1) | __ldg(w + nz_words + 1);
             }
-            const unsigned b = spread((busy[0] | busy[1]) & 0xFFFFu) |
-                               (spread((busy[1] | busy[2]) & 0xFFFFu) << 1);
-            free_bits |= (~b & (0xFFFFFFFFu >> (32u - n))) << done;
+            auto busy = [&](unsigned l, unsigned h) {  // of 16 columns, to the even bits
+                unsigned x = __funnelshift_r(l & in_lo, h & in_hi, static_cast<unsigned>(c - 1));
+                x = (x | (x >> 1)) & 0xFFFFu;
+                x = (x | (x << 8)) & 0x00FF00FFu;
+                x = (x | (x << 4)) & 0x0F0F0F0Fu;
+                x = (x | (x << 2)) & 0x33333333u;
+                return (x | (x << 1)) & 0x55555555u;
+            };
+            const unsigned b = busy(lo[0] | lo[1], hi[0] | hi[1]) |
+                               (busy(lo[1] | lo[2], hi[1] | hi[2]) << 1);
+            const unsigned f = ~b & (0xFFFFFFFFu >> (32u - n));
+            word |= f << done;
+            // the sampled cells among them: columns up to nx of rows up to ny
+            const int cells = J <= static_cast<unsigned>(ny) ? nx + 1 - c : 0;
+            if (cells > 0) sampled_free += __popc(cells >= 16 ? f : f & ((1u << (2 * cells)) - 1u));
             done += n;
             at += n;
             if (at == pair) {
@@ -304,9 +338,9 @@ __global__ void __launch_bounds__(256)
                 ++kk;
             }
         }
-        fr[g] = free_bits;
+        fr[g] = word;
     }
-    const unsigned free_here = __reduce_add_sync(0xffffffffu, __popc(free_bits));
+    const unsigned free_here = __reduce_add_sync(0xffffffffu, sampled_free);
     if (free_here >= kSparseFree && (threadIdx.x & 31) == 0) *sparse = 1;
 }
 
@@ -337,47 +371,45 @@ __global__ void export_kernel(const void* __restrict__ data, int storage, unsign
 
 cudaError_t launch_field(const float* rho, int nx, int ny, int nz, float K, hh_volume_s* vol,
                          cudaStream_t s) {
-    // 256 threads per block over (row pair, column), rows padded to whole
-    // warps; blockIdx.y picks the run of slice pairs: eight, or fewer where
-    // that leaves the chip with less than four blocks an SM
+    // eight warps of 32 columns a block, rows padded to whole warps; blockIdx.y
+    // picks the run of slice pairs: eight, or fewer where that leaves the chip
+    // with less than four blocks an SM
     const bool halo = vol->layout == HH_LAYOUT_ZPAIR;
     const dim3 block(256);
     auto grid_of = [&](int h, int& run) {
         const unsigned row_pairs = (ny + 2 * h + 1) / 2, pairs = (nz + 2 * h + 1) / 2;
-        const unsigned width = (nx + 2 * h + 31) / 32 * 32;
-        const unsigned blocks = (row_pairs * width + 255) / 256;
+        const unsigned blocks = (row_pairs * ((nx + 31) / 32) + 7) / 8;
         run = 8;
         while (run > 1 && blocks * ((pairs + run - 1) / run) < 608) run /= 2;
         return dim3(blocks, (pairs + run - 1) / run);
     };
     int run = 0;
-    const unsigned width = (nx + (halo ? 2 : 0) + 31) / 32 * 32;
     const dim3 grid = grid_of(halo ? 1 : 0, run);
     cudaError_t e = cudaSuccess;
     if (vol->storage == HH_STORE_FP32) {
         (halo ? field_kernel<0, 1> : field_kernel<0, 0>)<<<grid, block, 0, s>>>(
-            rho, nx, ny, nz, K, width, run, vol->row, vol->pair, vol->data, vol->nz_dev,
-            vol->nz_words, vol->sparse_dev, nullptr, vol->scales_dev);
+            rho, nx, ny, nz, K, run, vol->row, vol->pair, vol->data, vol->nz_dev,
+            vol->sparse_dev, nullptr, vol->scales_dev);
         count_launch();
     } else {
         e = cudaMemsetAsync(vol->max_dev, 0, 2 * sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
         int max_run = 0;
         const dim3 max_grid = grid_of(0, max_run);
-        field_kernel<1, 0><<<max_grid, block, 0, s>>>(rho, nx, ny, nz, K, (nx + 31) / 32 * 32,
-                                                      max_run, 0, 0, nullptr, nullptr, 0, nullptr,
-                                                      vol->max_dev, vol->scales_dev);
-        field_kernel<2, 1><<<grid, block, 0, s>>>(rho, nx, ny, nz, K, width, run, vol->row,
-                                                  vol->pair, vol->data, vol->nz_dev, vol->nz_words,
+        field_kernel<1, 0><<<max_grid, block, 0, s>>>(rho, nx, ny, nz, K, max_run, 0, 0, nullptr,
+                                                      nullptr, nullptr, vol->max_dev,
+                                                      vol->scales_dev);
+        field_kernel<2, 1><<<grid, block, 0, s>>>(rho, nx, ny, nz, K, run, vol->row,
+                                                  vol->pair, vol->data, vol->nz_dev,
                                                   vol->sparse_dev, vol->max_dev, vol->scales_dev);
         count_launch(2);
     }
     if (halo) {
-        const unsigned rows = (ny + 3) / 2 * 2, pairs = (nz + 3) / 2;
-        const unsigned words = static_cast<unsigned>((static_cast<size_t>(vol->pair) * pairs + 31) / 32);
-        free_mask_kernel<<<(words + 255) / 256, block, 0, s>>>(vol->nz_dev, vol->nz_words, rows,
-                                                               pairs, vol->row, vol->pair, words,
-                                                               vol->free_dev, vol->sparse_dev);
+        const unsigned pairs = (nz + 3) / 2;
+        const dim3 mgrid((vol->pair / 32 + 1 + 255) / 256, pairs);
+        free_mask_kernel<<<mgrid, block, 0, s>>>(
+            vol->nz_dev, vol->nz_words, nx, ny, pairs, vol->row, vol->pair,
+            1.0f / static_cast<float>(vol->row), vol->free_dev, vol->sparse_dev);
         count_launch();
     }
     return cudaGetLastError();

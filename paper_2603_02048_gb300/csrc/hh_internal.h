@@ -57,10 +57,10 @@ struct hh_volume_s {
     // (bit b & 31 of word b >> 5 for element b), set when the element's voxel
     // and its +1 neighbours on each axis hold no stored nonzero value, so that
     // a sample whose first corner is that voxel reads eight zeros. nz_dev: one
-    // bit per voxel, rows of nz_words words (bit I & 31 of word (K * (ny + 2) +
-    // J) * nz_words + (I >> 5)), set when the voxel holds a nonzero value. sparse_dev: nonzero when some
-    // stretch of the mask is worth testing (see free_mask_kernel). Null for
-    // LINEAR volumes.
+    // bit per grid column i, padded row J and slice K (bit i & 31 of word (K *
+    // rows + J) * nz_words + (i >> 5), rows = ny + 2 rounded up to even), set
+    // when the voxel holds a nonzero value. sparse_dev: nonzero when the mask is
+    // worth testing (see free_mask_kernel). Null for LINEAR volumes.
     size_t mask_off;    // bytes from data to free_dev
     unsigned nz_words;
     unsigned* free_dev;

@@ -142,3 +142,37 @@ def test_volume_beyond_4_gib(gpu):
     want = steps * h * c
     assert np.abs(turn - want).max() <= want * (8.2e-5 + 60 * 2.0**-24)
     vol.close()
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+@pytest.mark.parametrize("dims", [(70, 35, 50), (32, 46, 31), (33, 80, 47)])
+def test_rebuild_leaves_nothing_behind(gpu, dims, storage):
+    """Rebuilt from particles whose supports share no voxel (every density value
+    is then one product, the same in every run), after a build that filled the
+    whole volume and an empty one: bit for bit the volume and the rays of a
+    fresh build."""
+    hh, torch = gpu
+    g = np.random.default_rng(sum(dims))
+    h, kept = 1.0, []
+    for _ in range(400):
+        p = np.array([g.uniform(-2.0, n + 2.0) for n in dims])
+        if all(np.abs(p - q).max() > 4 * h + 1 for q in kept):
+            kept.append(p)
+    parts = np.concatenate([kept, g.uniform(0.5, 2.0, (len(kept), 1))], 1).astype(np.float32)
+    parts_t = torch.from_numpy(parts).cuda()
+    grid = hh.make_grid(dims, h, storage)
+    bg_t = torch.from_numpy(hi.checker_background()).cuda()
+    cams = f32([hi.orbit_camera(dims, az, 20.0, 48, 40, dist_factor=0.9) for az in (0.0, 215.0)])
+    params = f32(hi.params_rk4_fixed(dims, 0.5))
+    params["stepper"] = "euler"
+    fresh = hh.hh_build_index_field(parts_t, grid, 1e-4)
+    want4 = export_volume(hh, torch, fresh, dims)
+    want = gpu_trace(hh, torch, fresh, cams, params, bg_t)
+    full = torch.full((dims[0] * dims[1] * dims[2],), 0.7, device="cuda")
+    vol = hh.hh_volume_from_density(full, grid, 1.0)
+    hh.hh_volume_rebuild(vol, parts_t[:0].contiguous(), 1e-4)
+    assert not np.any(export_volume(hh, torch, vol, dims))
+    hh.hh_volume_rebuild(vol, parts_t, 1e-4)
+    assert np.array_equal(export_volume(hh, torch, vol, dims), want4)
+    for a, b in zip(gpu_trace(hh, torch, vol, cams, params, bg_t), want):
+        assert all(np.array_equal(a[n], b[n]) for n in a)
