@@ -666,11 +666,12 @@ __device__ __forceinline__ void ray_begin(const VolArgs& V, const float* __restr
 }
 
 // One step of Eq. 16 (or RK4) with the Eq. 18 (or fixed) step length.
-// Returns true when the step leaves the box: then ep / ed hold the exit
-// point on the face and the new direction.
+// Returns true when the step leaves the box: then R.hi and R.d, of no further
+// use to the march, hold the exit point on the face and the new direction (six
+// registers that the loop need not carry).
 template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR, bool MASK>
-__device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restrict__ vol, RayState& R,
-                                         float3& ep, float3& ed) {
+__device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restrict__ vol,
+                                         RayState& R) {
     const float B = V.bias;
     const float3 wr = R.wr, d = R.d;
     const float3 C = R.c;
@@ -751,8 +752,8 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
     if (outside(V, P)) {
         const float3 h0 = make_float3(ohi.x - B, ohi.y - B, ohi.z - B);  // exact
         const float tau = exit_fraction(V, h0, olo, inc);
-        ep = h0 + fma3(tau, inc, olo);
-        ed = wr + dnew;
+        R.hi = h0 + fma3(tau, inc, olo);
+        R.d = wr + dnew;
         R.flags |= HH_FLAG_EXITED;
         return true;
     }
@@ -764,14 +765,14 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
 // free-corner mask or the one that does not.
 template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
 __device__ __forceinline__ void ray_march(const VolArgs& V, const void* __restrict__ vol,
-                                          unsigned sparse, RayState& R, float3& ep, float3& ed) {
+                                          unsigned sparse, RayState& R) {
     if (sparse) {
         while (R.k < V.max_steps &&
-               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, vol, R, ep, ed)) {
+               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, vol, R)) {
         }
     } else {
         while (R.k < V.max_steps &&
-               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, vol, R, ep, ed)) {
+               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, vol, R)) {
         }
     }
 }
@@ -785,8 +786,9 @@ __device__ __forceinline__ uint8_t to_u8(float v) {
 // missed reports the eye and its primary direction; one that ran out of
 // steps reports its current state (MAXSTEPS).
 __device__ __forceinline__ void ray_end(const VolArgs& V, const ViewArgs& C, int px, int py,
-                                        const RayState& R, float3 ep, float3 ed) {
+                                        const RayState& R) {
     uint32_t flags = R.flags;
+    float3 ep = R.hi, ed = R.d;  // of a ray that exited
     if (!(flags & HH_FLAG_HIT)) {
         ep = C.eye;
         ed = R.wr;
@@ -834,11 +836,10 @@ __global__ void __launch_bounds__(128, march_blocks(STEPPER))
     const int py = blockIdx.y * 8 + (warp >> 1) * 4 + ty;
     if (px >= C.W || py >= C.H) return;
     RayState R;
-    float3 ep = C.eye, ed = C.eye;
     ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
     if (R.flags & HH_FLAG_HIT)
-        ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, __ldg(V.sparse), R, ep, ed);
-    ray_end(V, C, px, py, R, ep, ed);
+        ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, __ldg(V.sparse), R);
+    ray_end(V, C, px, py, R);
 }
 
 // View and place (column, row of tiles) of batch tile t: from the order table
@@ -935,11 +936,10 @@ __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
             const int px = (tx << tile_w_log2) + lx, py = ty * (32 >> tile_w_log2) + ly;
             if (px < C.W && py < C.H) {
                 RayState R;
-                float3 ep = make_float3(0.0f, 0.0f, 0.0f), ed = ep;
                 ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
                 if (R.flags & HH_FLAG_HIT)
-                    ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, sparse, R, ep, ed);
-                ray_end(V, C, px, py, R, ep, ed);
+                    ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, sparse, R);
+                ray_end(V, C, px, py, R);
             }
         }
     }
@@ -947,7 +947,6 @@ __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
     bool done = false, have = false;
     int vi = 0, px = 0, py = 0;
     RayState R;
-    float3 ep = make_float3(0.0f, 0.0f, 0.0f), ed = ep;
     for (;;) {
         const unsigned free_mask = __ballot_sync(FULL, !have);
         if (!done && __popc(free_mask) >= refill_min) {
@@ -978,7 +977,7 @@ __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
                     if (px < C.W && py < C.H) {
                         ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
                         if ((R.flags & HH_FLAG_HIT) && V.max_steps > 0) have = true;
-                        else ray_end(V, C, px, py, R, ep, ed);
+                        else ray_end(V, C, px, py, R);
                     }
                 }
                 pos += min(avail, __popc(todo));
@@ -991,10 +990,10 @@ __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
         }
         if (have) {
             const bool left =
-                sparse ? ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, V.vol, R, ep, ed)
-                       : ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, V.vol, R, ep, ed);
+                sparse ? ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, V.vol, R)
+                       : ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, V.vol, R);
             if (left || R.k >= V.max_steps) {
-                ray_end(V, views[vi], px, py, R, ep, ed);
+                ray_end(V, views[vi], px, py, R);
                 have = false;
             }
         }
@@ -1047,6 +1046,9 @@ struct alignas(16) WorkerWarp {
     unsigned sparse;
     int view_begin, n_views, n_tiles;
     int view_first, view_end;  // job-relative tiles of the view held
+    unsigned long long idle_since;
+    unsigned backoff;          // ns
+    int counted_idle;
 };
 
 // Resident 256-thread blocks per SM of the serving worker: as the batched
@@ -1066,18 +1068,20 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
     ViewArgs& C = S.view;
     const int tile_w_log2 = W.tile_w == 16 ? 4 : (W.tile_w == 8 ? 3 : 2);
     const int tile_h = 32 >> tile_w_log2;
-    int lx, ly;
-    tile_pixel(lane, tile_w_log2, lx, ly);
     const char* views = static_cast<const char*>(W.views);
     constexpr int kWords = sizeof(ViewArgs) / sizeof(unsigned);
     int j = ld_acquire_int(W.first_open);
     int have_job = -1;
     unsigned t = 0;  // this warp's claimed tile of job j (valid while have_job == j)
     bool claimed_next = false;
-    unsigned long long idle_since = 0;
-    unsigned backoff = 1000;
-    bool counted_idle = false;
-    if (lane == 0) atomicAdd(W.started_warps, 1);
+    // lane 0's alone: since when the warp has been idle, whether it counts so
+    if (lane == 0) {
+        S.idle_since = 0;
+        S.backoff = 1000;
+        S.counted_idle = 0;
+        atomicAdd(W.started_warps, 1);
+    }
+    __syncwarp();
     for (;;) {
         if (j != have_job) {
             // wait for job j: published, then written (both bounded in time)
@@ -1116,9 +1120,9 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
                 int leave = 0;
                 if (lane == 0) {
                     const unsigned long long now = global_ns();
-                    if (idle_since == 0) idle_since = now;
-                    if (!counted_idle && now - idle_since > W.idle_ns) {
-                        counted_idle = true;
+                    if (S.idle_since == 0) S.idle_since = now;
+                    if (!S.counted_idle && now - S.idle_since > W.idle_ns) {
+                        S.counted_idle = 1;
                         // all warps that have started are idle: the launch leaves
                         // (a block that starts later sees the flag and leaves too)
                         if (atomicAdd(W.idle_warps, 1) + 1 == ld_acquire_int(W.started_warps))
@@ -1127,8 +1131,10 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
                     leave = ld_acquire_int(W.leave);
                 }
                 if (__shfl_sync(FULL, leave, 0)) break;
-                __nanosleep(backoff);
-                backoff = min(backoff * 2u, 32000u);
+                __nanosleep(S.backoff);
+                __syncwarp();
+                if (lane == 0) S.backoff = min(S.backoff * 2u, 32000u);
+                __syncwarp();
                 j = max(j, ld_acquire_int(W.first_open));
                 continue;
             }
@@ -1136,14 +1142,12 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
                 ++j;
                 continue;
             }
-            idle_since = 0;
-            backoff = 1000;
-            if (counted_idle) {
-                if (lane == 0) atomicSub(W.idle_warps, 1);
-                counted_idle = false;
-            }
             __syncwarp();
             if (lane == 0) {
+                S.idle_since = 0;
+                S.backoff = 1000;
+                if (S.counted_idle) atomicSub(W.idle_warps, 1);
+                S.counted_idle = 0;
                 const ServeJob* e = W.jobs + j;
                 S.vol = __ldcg(reinterpret_cast<const unsigned long long*>(&e->vol));
                 S.scales = __ldcg(reinterpret_cast<const unsigned long long*>(&e->scales));
@@ -1192,15 +1196,16 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
         }
         const int local = ti - S.view_first;
         const int ty = local / C.tiles_x, tx = local - ty * C.tiles_x;
+        int lx, ly;
+        tile_pixel(lane, tile_w_log2, lx, ly);
         const int px = (tx << tile_w_log2) + lx, py = ty * tile_h + ly;
         if (px < C.W && py < C.H) {
             RayState R;
-            float3 ep = make_float3(0.0f, 0.0f, 0.0f), ed = ep;
-            ray_begin<ADAPTIVE>(V, reinterpret_cast<const float*>(S.scales), C, px, py, R);
+                    ray_begin<ADAPTIVE>(V, reinterpret_cast<const float*>(S.scales), C, px, py, R);
             if (R.flags & HH_FLAG_HIT)
                 ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>(
-                    V, reinterpret_cast<const void*>(S.vol), S.sparse, R, ep, ed);
-            ray_end(V, C, px, py, R, ep, ed);
+                    V, reinterpret_cast<const void*>(S.vol), S.sparse, R);
+            ray_end(V, C, px, py, R);
         }
         // count the tile (release: its outputs are ordered before the count,
         // so the warp that sees the count reach n_tiles sees every tile) and
