@@ -53,9 +53,14 @@ namespace {
 constexpr float kPi = 3.14159265358979323846f;
 
 // Resident 128-thread blocks per SM the single-view march kernels are compiled
-// for: 8 leaves 64 registers a thread (Eq. 16; 9 or 10 measured the same, or
-// slower where they spill), 6 leaves 80 (RK4).
-constexpr int march_blocks(int stepper) { return stepper == HH_STEP_RK4 ? 6 : 8; }
+// for. Eq. 16: 8, i.e. at most 64 registers a thread (9 or 10 measured the same,
+// or slower where they spill). RK4: 6 (80 registers) on FP16, 5 (102) on FP32
+// storage, whose four samples a step otherwise spill (256^3 720p view 2514
+// against 2446 us, 64^3 128x128 164 against 140; FP16 1080p view 964 against 1014
+// with 5).
+constexpr int march_blocks(int storage, int stepper) {
+    return stepper != HH_STEP_RK4 ? 8 : storage == HH_STORE_FP32 ? 5 : 6;
+}
 // Resident 256-thread blocks per SM of the persistent batched kernel. More
 // warps hide more of the L2 latency as long as the step does not spill. Tile at
 // a time, FP16: 5 blocks (48 registers) against 4, 8 views of the 256^3 volume
@@ -827,7 +832,7 @@ __device__ __forceinline__ void ray_end(const VolArgs& V, const ViewArgs& C, int
 // One view, one thread per pixel: a block of 128 threads covers 16x8 pixels,
 // each warp an 8x4 tile.
 template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
-__global__ void __launch_bounds__(128, march_blocks(STEPPER))
+__global__ void __launch_bounds__(128, march_blocks(STORAGE, STEPPER))
     march_kernel(const VolArgs V, const ViewArgs C) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int tx, ty;
