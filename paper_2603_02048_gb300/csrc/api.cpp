@@ -150,8 +150,8 @@ hh_status new_volume(const hh_grid* g, hh_volume* out) {
     v->storage = g->storage;
     v->h_kernel = g->h_kernel;
     v->layout = HH_LAYOUT_ZPAIR;
-    v->row = zpair_row(g->nx);
-    v->pair = zpair_pair(g->nx, g->ny);
+    v->row = zpair_row(g->nx, g->storage);
+    v->pair = zpair_pair(v->row, g->ny);
     const size_t voxel_bytes = g->storage == HH_STORE_FP32 ? 16 : 8;
     v->bytes = stored_voxels(g) * voxel_bytes;
     // the free-corner mask, its build scratch (a bit per element and voxel)

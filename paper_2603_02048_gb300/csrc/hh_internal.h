@@ -30,18 +30,23 @@
 //          takes 333 and 1604, but its lines of eight voxels in a row spread a
 //          cell over more of them (32 views of a 512^3 FP16 volume: 11.1 ms
 //          against 10.0, and 10.1 for the bricks).
-//          row = 12 and pair = 2 (mod 16): the eight corners of any cell lie
-//          in eight different 16-byte L1 bank groups (8-byte ones on FP16
-//          storage), and so do the cells around it as far as that goes; of ten
-//          residue pairs this one was the fastest on the 512^3 views (10.0
-//          against 10.1-10.8 ms) and no slower on the others.
+//          The strides' residues spread a warp's corner load, the same corner
+//          of 32 neighbouring cells, over the L1's bank groups and tag banks
+//          (the start of the next row or pair of slices must not fold onto this
+//          one's). Measured over paddings of 0 to 42 elements: pair = 2 (mod
+//          16), and row = 6 (mod 8) on FP32 storage (1080p view of a dense 256^3
+//          volume 365 us; 376 at 12 (mod 16), 470 at 8), 12 (mod 16) on FP16 (32
+//          views of a 512^3 volume 9.13 ms against 9.15 to 9.60).
 enum { HH_LAYOUT_LINEAR = 0, HH_LAYOUT_ZPAIR = 1 };
 
 // ZPAIR strides in elements: of a row, and of a pair of slices. (A grid within
 // the size limit of the entry points has less than 2^32 elements.)
-inline unsigned zpair_row(int nx) { return (2u * static_cast<unsigned>(nx) + 7u) / 16u * 16u + 12u; }
-inline unsigned zpair_pair(int nx, int ny) {
-    return (zpair_row(nx) * (static_cast<unsigned>(ny) + 2u) + 13u) / 16u * 16u + 2u;
+inline unsigned zpair_row(int nx, int storage) {
+    const unsigned n = 2u * (static_cast<unsigned>(nx) + 2u);
+    return storage == HH_STORE_FP32 ? (n + 1u) / 8u * 8u + 6u : (n + 3u) / 16u * 16u + 12u;
+}
+inline unsigned zpair_pair(unsigned row, int ny) {
+    return (row * (static_cast<unsigned>(ny) + 2u) + 13u) / 16u * 16u + 2u;
 }
 
 struct hh_volume_s {
