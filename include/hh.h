@@ -286,9 +286,11 @@ typedef struct {
     int tile_order;    /* order in which warps take tiles: 0 = view after view,
                           row by row; 1 = the tiles of all views interleaved
                           by their relative row, so every view sweeps the
-                          volume top to bottom at once (views at similar
-                          elevations then share the bricks in L2: 17 % less
-                          DRAM traffic on the 512^3 32-view batch).       */
+                          volume top to bottom at once, the top quarter
+                          last, beside the bottom (views at similar
+                          elevations then share the volume's lines in L2:
+                          17 % less DRAM traffic on the 512^3 32-view
+                          batch).                                         */
     int tile_group;    /* 0 = each warp takes its own next tile; 1 = a block
                           takes one tile per warp at once (consecutive tiles,
                           neighbours in a view) so that its warps march them

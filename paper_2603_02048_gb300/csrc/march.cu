@@ -829,16 +829,27 @@ __device__ __forceinline__ void ray_end(const VolArgs& V, const ViewArgs& C, int
     if (C.flags) C.flags[pix] = flags;
 }
 
+// Row of tiles taken i-th of n, from row mid outwards: mid, mid + 1, mid - 1, ...,
+// then the rest of the longer side.
+__device__ __forceinline__ int row_from(int i, int n, int mid) {
+    if (i <= 2 * min(mid, n - 1 - mid)) return mid + ((i & 1) ? (i + 1) >> 1 : -(i >> 1));
+    return mid < n - 1 - mid ? i : n - 1 - i;
+}
+
 // One view, one thread per pixel: a block of 128 threads covers 16x8 pixels,
-// each warp an 8x4 tile.
+// each warp an 8x4 tile. Blocks start with the row of tiles that sees the
+// volume's centre and go outwards: the rays get shorter, so that the launch
+// does not end on a few long ones (720p view of a 192x160x224 turbulence volume
+// 180 us top to bottom, 166 so; 641x363 RK4 view 94 against 85; 1080p view of
+// the 256^3 plume 295 against 285).
 template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
 __global__ void __launch_bounds__(128, march_blocks(STORAGE, STEPPER))
-    march_kernel(const VolArgs V, const ViewArgs C) {
+    march_kernel(const VolArgs V, const ViewArgs C, const int mid) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int tx, ty;
     tile_pixel(lane, 3, tx, ty);
     const int px = blockIdx.x * 16 + (warp & 1) * 8 + tx;
-    const int py = blockIdx.y * 8 + (warp >> 1) * 4 + ty;
+    const int py = row_from(blockIdx.y, gridDim.y, mid) * 8 + (warp >> 1) * 4 + ty;
     if (px >= C.W || py >= C.H) return;
     RayState R;
     ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
@@ -1242,10 +1253,18 @@ template <int STORAGE, int STEPPER, bool ADAPTIVE>
 void launch_one(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
     const dim3 block(128);
     const dim3 grid((C.W + 15) / 16, (C.H + 7) / 8);
+    // row of blocks that sees the volume's centre (the middle one if it is behind
+    // the camera)
+    const float o[3] = {0.5f * V.nx - C.eye.x, 0.5f * V.ny - C.eye.y, 0.5f * V.nz - C.eye.z};
+    const float ahead = C.f.x * o[0] + C.f.y * o[1] + C.f.z * o[2];
+    const float up = C.u.x * o[0] + C.u.y * o[1] + C.u.z * o[2];
+    float row = 0.5f * C.H;
+    if (ahead > 0.0f) row = (C.b0 - up / ahead) / C.s;
+    const int mid = static_cast<int>(fminf(fmaxf(row, 0.0f), C.H - 1.0f)) / 8;
     if (addr_any(V))
-        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY><<<grid, block, 0, s>>>(V, C);
+        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY><<<grid, block, 0, s>>>(V, C, mid);
     else
-        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_BASE><<<grid, block, 0, s>>>(V, C);
+        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_BASE><<<grid, block, 0, s>>>(V, C, mid);
 }
 
 // Calls F<STORAGE, STEPPER, ADAPTIVE>::run(args...) for the runtime choice.
@@ -1483,7 +1502,12 @@ void drop_graph(hh_batch b) {
 
 // The interleaved tile order (tile_order 1): the tiles of all views sorted by
 // their relative row in their view (then by view, then by column), so that
-// every view sweeps the volume top to bottom at the same time.
+// every view sweeps the volume top to bottom at the same time. The top quarter,
+// whose rays are short, is not taken first but beside the bottom quarter, in
+// mirrored order, so that the launch ends on its shortest rays (8 views of a
+// 256^3 FP16 volume 1054 -> 1033 us, 12 uneven ones of 384^3 2293 -> 2275; from
+// the middle outwards 1034, but 2309: two sweeps share fewer lines in L2; 32
+// views of 512^3 the same 9.14 ms).
 std::vector<uint2> interleaved_order(const std::vector<hh::ViewArgs>& v, int tile_w) {
     struct Key {
         double k;
@@ -1495,7 +1519,9 @@ std::vector<uint2> interleaved_order(const std::vector<hh::ViewArgs>& v, int til
         const int tiles_y = (v[i].H + tile_h - 1) / tile_h;
         for (int ty = 0; ty < tiles_y; ++ty)
             for (int tx = 0; tx < v[i].tiles_x; ++tx)
-                keys.push_back({(ty + 0.5) / tiles_y, static_cast<uint32_t>(i),
+                keys.push_back({ty + 0.5 < 0.25 * tiles_y ? 1.0 - (ty + 0.5) / tiles_y
+                                                          : (ty + 0.5) / tiles_y,
+                                static_cast<uint32_t>(i),
                                 static_cast<uint32_t>(ty) << 16 | static_cast<uint32_t>(tx)});
     }
     std::stable_sort(keys.begin(), keys.end(), [](const Key& x, const Key& y) { return x.k < y.k; });
