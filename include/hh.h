@@ -230,10 +230,12 @@ hh_status hh_build_index_field_noalloc(const hh_particles* particles, const hh_g
 hh_status hh_volume_export(hh_volume vol, float* dst_dev, void* stream);
 
 /* Grid, FP16 scales (1 for FP32 storage) and device bytes of a volume's
- * packed field (bookkeeping; no paper passage; the same allocation also holds
- * a free-corner mask, one bit per voxel, and its build scratch, a word per
- * stored column and 16 slices: under 5 % more). Synchronises `stream` to read
- * the scales. Any output may be NULL. */
+ * packed field, the grid and its halo with every axis padded to even
+ * (bookkeeping; no paper passage; the same allocation also holds the padding
+ * of its rows, at most 14 elements for two rows, a free-corner mask, one bit
+ * per element, and its build scratch, one bit per voxel: at 256^3 2 % more on
+ * FP32 storage, 5 % on FP16). Synchronises `stream` to read the scales. Any
+ * output may be NULL. */
 hh_status hh_volume_info(hh_volume vol, hh_grid* grid, float* s_n, float* s_g, size_t* bytes,
                          void* stream);
 
