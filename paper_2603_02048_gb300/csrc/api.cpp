@@ -247,7 +247,7 @@ hh_status volume_from(const float* rho_dev, const hh_grid* grid, float K, cudaSt
     hh_volume v = nullptr;
     hh_status st = new_volume(grid, &v);
     if (st != HH_OK) return st;
-    cudaError_t e = launch_field(rho_dev, grid->nx, grid->ny, grid->nz, K, v, s);
+    cudaError_t e = launch_field(rho_dev, grid->nx, grid->ny, grid->nz, K, v, false, s);
     if (e != cudaSuccess) {
         drop_volume(v);
         return cuda_fail(e, "field kernel launch");
@@ -339,7 +339,7 @@ hh_status hh_splat_density(const hh_particles* particles, const hh_grid* grid, f
     if (!rho_dev) return fail(HH_ERR_INVALID_ARG, "rho_dev is NULL");
     cudaError_t e = launch_splat(reinterpret_cast<const float4*>(particles->xyzm_dev), particles->n,
                                  grid->nx, grid->ny, grid->nz, grid->h_kernel, rho_dev,
-                                 as_stream(stream));
+                                 nullptr, as_stream(stream));
     if (e != cudaSuccess) return cuda_fail(e, "splat launch");
     return ok();
 }
@@ -405,9 +405,9 @@ hh_status hh_volume_rebuild(hh_volume vol, const hh_particles* particles, float 
         src = vol->sorted_dev;
     }
     cudaError_t e = launch_splat(src, particles->n, vol->nx, vol->ny, vol->nz, vol->h_kernel,
-                                 vol->rho_dev, s);
+                                 vol->rho_dev, vol->max_dev, s);
     if (e != cudaSuccess) return cuda_fail(e, "splat launch");
-    e = launch_field(vol->rho_dev, vol->nx, vol->ny, vol->nz, K_gd, vol, s);
+    e = launch_field(vol->rho_dev, vol->nx, vol->ny, vol->nz, K_gd, vol, true, s);
     if (e != cudaSuccess) return cuda_fail(e, "field kernel launch");
     return ok();
 }

@@ -36,6 +36,15 @@
 // warp whose lanes all sample zero skips it); every step is still taken with
 // the values the general branch would compute, so the results do not depend
 // on the skip.
+//
+// What bounds it: instruction issue and the L1 data pipe, of which a dense
+// volume takes most (a load costs a cycle per distinct 16-byte unit in the
+// fullest of eight banks). 1080p view of the 256^3 FP32 plume at h_max: 66 % of
+// the issue slots, 65 % of the pipe; eight 720p views of it on FP16: 80 and 71 %;
+// 32 views of a 512^3 FP16 volume: 86 % of the pipe. RK4 with few rays is bound
+// by the four serial samples a step, ~340 cycles each. Against 2x2x2 bricks,
+// scalar state and IEEE approximations the step took these launches from 360 to
+// 285, 1227 to 1035 us and 10.1 to 9.15 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -841,20 +850,24 @@ __device__ __forceinline__ int row_from(int i, int n, int mid) {
 // volume's centre and go outwards: the rays get shorter, so that the launch
 // does not end on a few long ones (720p view of a 192x160x224 turbulence volume
 // 180 us top to bottom, 166 so; 641x363 RK4 view 94 against 85; 1080p view of
-// the 256^3 plume 295 against 285).
+// the 256^3 plume 295 against 285). Its blocks never release_next(): those of
+// another view behind it would gather on the SMs that empty first (the RK4 view,
+// launches back to back: 87.5 us, without 62.1, launched as ordinary ones 64.6).
 template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
 __global__ void __launch_bounds__(128, march_blocks(STORAGE, STEPPER))
     march_kernel(const VolArgs V, const ViewArgs C, const int mid) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int tx, ty;
     tile_pixel(lane, 3, tx, ty);
+    // (every load of the volume's depends on the pixel)
+    asm volatile("griddepcontrol.wait;" : "+r"(tx), "+r"(ty) :: "memory");
     const int px = blockIdx.x * 16 + (warp & 1) * 8 + tx;
     const int py = row_from(blockIdx.y, gridDim.y, mid) * 8 + (warp >> 1) * 4 + ty;
     if (px >= C.W || py >= C.H) return;
     RayState R;
-    ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
+    ray_begin<ADAPTIVE>(V, after_wait(V.scales), C, px, py, R);
     if (R.flags & HH_FLAG_HIT)
-        ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, __ldg(V.sparse), R);
+        ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, __ldg(after_wait(V.sparse)), R);
     ray_end(V, C, px, py, R);
 }
 
@@ -1262,9 +1275,9 @@ void launch_one(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
     if (ahead > 0.0f) row = (C.b0 - up / ahead) / C.s;
     const int mid = static_cast<int>(fminf(fmaxf(row, 0.0f), C.H - 1.0f)) / 8;
     if (addr_any(V))
-        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY><<<grid, block, 0, s>>>(V, C, mid);
+        launch_next(march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>, grid, block, s, V, C, mid);
     else
-        march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_BASE><<<grid, block, 0, s>>>(V, C, mid);
+        launch_next(march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_BASE>, grid, block, s, V, C, mid);
 }
 
 // Calls F<STORAGE, STEPPER, ADAPTIVE>::run(args...) for the runtime choice.

@@ -93,10 +93,10 @@ extern "C" hh_status hh_build_index_field_noalloc(const hh_particles* particles,
     hh_status st = static_scratch(&s);
     if (st != HH_OK) return st;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    // launch_splat clears the density (cudaMemsetAsync) before accumulating.
+    // launch_splat clears the density before accumulating.
     cudaError_t e = hh::launch_splat(reinterpret_cast<const float4*>(particles->xyzm_dev),
                                      particles->n, grid->nx, grid->ny, grid->nz, grid->h_kernel,
-                                     s->rho, cs);
+                                     s->rho, nullptr, cs);
     if (e != cudaSuccess) return hh::cuda_fail(e, "splat launch");
     hh_volume_s out{};
     out.nx = grid->nx;
@@ -109,7 +109,7 @@ extern "C" hh_status hh_build_index_field_noalloc(const hh_particles* particles,
     out.bytes = nvox * 16;
     out.scales_dev = s->scales;
     out.max_dev = s->max;
-    e = hh::launch_field(s->rho, grid->nx, grid->ny, grid->nz, K_gd, &out, cs);
+    e = hh::launch_field(s->rho, grid->nx, grid->ny, grid->nz, K_gd, &out, false, cs);
     if (e != cudaSuccess) return hh::cuda_fail(e, "field kernel launch");
     return hh::ok();
 }

@@ -69,6 +69,29 @@ __device__ __forceinline__ void footprint(float x, float reach, int n, int& lo, 
     hi = min(n - 1, (int)floorf(b));
 }
 
+// Clears n floats, sixteen a thread in 16-byte stores, and the two words at
+// max_bits (nullable). A kernel and not a memset so that the splat's blocks can
+// start, and read their particles, behind it (launch_next): the density of
+// 262,144 particles on 256^3 103.3 against 99.1 us. What bounds it: L2 writes. It is launched as an ordinary kernel: the particles are complete
+// before it starts, so the splat may read them before it ends.
+__global__ void __launch_bounds__(256) zero_kernel(float* __restrict__ p, size_t n,
+                                                   unsigned* __restrict__ max_bits) {
+    release_next();
+    const size_t head = min(n, (16u - (reinterpret_cast<size_t>(p) & 15u)) / 4u & 3u);
+    float4* const body = reinterpret_cast<float4*>(p + head);
+    const size_t n4 = (n - head) / 4, done = head + 4 * n4;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const size_t i = (static_cast<size_t>(blockIdx.x) * 4 + k) * blockDim.x + threadIdx.x;
+        if (i < n4) body[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < head) p[threadIdx.x] = 0.0f;
+        if (threadIdx.x < n - done) p[done + threadIdx.x] = 0.0f;
+        if (max_bits && threadIdx.x < 2) max_bits[threadIdx.x] = 0u;
+    }
+}
+
 constexpr int kParticlesPerWarp = 4;  // of splat_warp_kernel
 
 template <int PPW>  // particles per warp: 32 / PPW lanes each
@@ -84,6 +107,8 @@ __global__ void __launch_bounds__(256) splat_warp_kernel(const float4* __restric
         ((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * PPW + lane / LPP;
     if (p >= n) return;
     const float4 q = __ldg(parts + p);
+    await_previous();  // the density is cleared
+    release_next();
     int x0, x1, y0, y1, z0, z1;
     footprint(q.x, 2.0f * h, nx, x0, x1);
     footprint(q.y, 2.0f * h, ny, y0, y1);
@@ -186,6 +211,8 @@ __global__ void __launch_bounds__(256) splat_box_kernel(const float4* __restrict
                           (32 / LPP) + lane / LPP;
     if (p >= n) return;
     const float4 q = __ldg(parts + p);
+    await_previous();  // the density is cleared
+    release_next();
     const float reach = 2.0f * h;
     const float inv_2h = 0.5f * inv_h;
     const int sx = box_start<N>(q.x, reach, nx), sy = box_start<N>(q.y, reach, ny),
@@ -387,12 +414,17 @@ cudaError_t launch_bin_particles(const float4* xyzm, int64_t n, int nx, int ny, 
 }
 
 cudaError_t launch_splat(const float4* xyzm, int64_t n, int nx, int ny, int nz, float h,
-                         float* rho, cudaStream_t s) {
+                         float* rho, unsigned* max_bits, cudaStream_t s) {
     const size_t nvox = static_cast<size_t>(nx) * ny * nz;
-    cudaError_t e = cudaMemsetAsync(rho, 0, nvox * sizeof(float), s);
-    if (e != cudaSuccess) return e;
-    if (n == 0) return cudaSuccess;
+    if (n == 0) {
+        cudaError_t e = cudaMemsetAsync(rho, 0, nvox * sizeof(float), s);
+        if (e == cudaSuccess && max_bits) e = cudaMemsetAsync(max_bits, 0, 2 * sizeof(unsigned), s);
+        return e;
+    }
     const int threads = 256;
+    zero_kernel<<<static_cast<unsigned>(nvox / (16 * threads) + 1), threads, 0, s>>>(rho, nvox,
+                                                                                   max_bits);
+    count_launch();
     auto blocks = [&](int ppw) {  // of warps with ppw particles each
         return static_cast<unsigned>(((n + ppw - 1) / ppw * 32 + threads - 1) / threads);
     };
@@ -402,7 +434,7 @@ cudaError_t launch_splat(const float4* xyzm, int64_t n, int nx, int ny, int nz, 
     int e2 = 0;
     const bool unit = hd < 0.5 || std::frexp(hd, &e2) == 0.5;
     auto box = [&](auto kernel, int lanes) {
-        kernel<<<blocks(32 / lanes), threads, 0, s>>>(xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
+        launch_next(kernel, blocks(32 / lanes), threads, s, xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
     };
     // the smallest box that holds the support (4h slots an axis)
     if (hd <= 1.0)
@@ -418,8 +450,7 @@ cudaError_t launch_splat(const float4* xyzm, int64_t n, int nx, int ny, int nz, 
     else if (hd <= 4.0)
         box(splat_box_kernel<16, 16, false>, 16);
     else
-        splat_warp_kernel<kParticlesPerWarp><<<blocks(kParticlesPerWarp), threads, 0, s>>>(
-            xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
+        launch_next(splat_warp_kernel<kParticlesPerWarp>, blocks(kParticlesPerWarp), threads, s, xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
     count_launch();
     return cudaGetLastError();
 }
