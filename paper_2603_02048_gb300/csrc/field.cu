@@ -141,6 +141,12 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
         a1 = at(r1, min(k, nz - 1));
     }
     float mn = 0.0f, mg = 0.0f;
+    // the max pass scales the largest x and y differences once, at the end (max and
+    // the multiplication by 1/2 commute), and walks two pairs at once: 256^3 FP16
+    // build 183.7 against 181.5 us, 512^3 1564 against 1557
+    float mx = 0.0f, my0 = 0.0f, my1 = 0.0f;
+    const float kx = MODE == 1 ? 1.0f : fx, ky0 = MODE == 1 ? 1.0f : fy0, ky1 = MODE == 1 ? 1.0f : fy1;
+#pragma unroll(MODE == 1 ? 2 : 1)
     for (int kk = kk0; kk < kk1; ++kk) {
         const int K0 = 2 * kk - H, K1 = K0 + 1;  // grid slices of the pair
         const int s0 = min(max(K0, 0), nz - 1), s1 = min(K1, nz - 1), sn = min(K1 + 1, nz - 1);
@@ -166,28 +172,26 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
         {
             const size_t z = static_cast<size_t>(s0) * sz;
             const float oa = dn_of(ra + z), od = dn_of(rd + z);
-            v00.gx = (dn_of(r0 + z + xh) - dn_of(r0 + z + xl)) * fx;
-            v10.gx = (dn_of(r1 + z + xh) - dn_of(r1 + z + xl)) * fx;
-            v00.gy = ((first_row ? od : a1) - oa) * fy0;
-            v10.gy = (od - (last_row ? oa : a0)) * fy1;
+            v00.gx = (dn_of(r0 + z + xh) - dn_of(r0 + z + xl)) * kx;
+            v10.gx = (dn_of(r1 + z + xh) - dn_of(r1 + z + xl)) * kx;
+            v00.gy = ((first_row ? od : a1) - oa) * ky0;
+            v10.gy = (od - (last_row ? oa : a0)) * ky1;
         }
         {
             const size_t z = static_cast<size_t>(s1) * sz;
             const float oa = dn_of(ra + z), od = dn_of(rd + z);
-            v01.gx = (dn_of(r0 + z + xh) - dn_of(r0 + z + xl)) * fx;
-            v11.gx = (dn_of(r1 + z + xh) - dn_of(r1 + z + xl)) * fx;
-            v01.gy = ((first_row ? od : b1) - oa) * fy0;
-            v11.gy = (od - (last_row ? oa : b0)) * fy1;
+            v01.gx = (dn_of(r0 + z + xh) - dn_of(r0 + z + xl)) * kx;
+            v11.gx = (dn_of(r1 + z + xh) - dn_of(r1 + z + xl)) * kx;
+            v01.gy = ((first_row ? od : b1) - oa) * ky0;
+            v11.gy = (od - (last_row ? oa : b0)) * ky1;
         }
         if (MODE == 1) {
-            auto peak = [&](const Voxel& v) {
-                mn = fmaxf(mn, fabsf(v.dn));
-                mg = fmaxf(mg, fmaxf(fabsf(v.gx), fmaxf(fabsf(v.gy), fabsf(v.gz))));
-            };
-            peak(v00);
-            peak(v10);
-            peak(v01);
-            peak(v11);
+            auto peak = [](float m, float a, float b) { return fmaxf(m, fmaxf(fabsf(a), fabsf(b))); };
+            mn = peak(peak(mn, a0, a1), b0, b1);
+            mx = peak(peak(mx, v00.gx, v10.gx), v01.gx, v11.gx);
+            my0 = peak(my0, v00.gy, v01.gy);
+            my1 = peak(my1, v10.gy, v11.gy);
+            mg = peak(peak(mg, v00.gz, v10.gz), v01.gz, v11.gz);
         } else if (H == 0) {
             if (valid) {
                 const size_t o = (static_cast<size_t>(K0) * ny + J0) * nx + i;
@@ -253,6 +257,7 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
         a1 = n1;
     }
     if (MODE == 1) {  // block maximum, then one atomic per block
+        mg = fmaxf(fmaxf(mg, mx * fx), fmaxf(my0 * fy0, my1 * fy1));
         for (int d = 16; d > 0; d >>= 1) {
             mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, d));
             mg = fmaxf(mg, __shfl_xor_sync(0xffffffffu, mg, d));
