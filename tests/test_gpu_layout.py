@@ -116,6 +116,34 @@ def test_march_with_and_without_mask(gpu, oracle_lib, dims, dense, storage, step
     vol.close()
 
 
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+@pytest.mark.parametrize("gap", [1, 2, 5, 9])
+def test_march_in_and_out_of_free_cells(gpu, oracle_lib, storage, gap):
+    """Shells of matter with gaps of `gap` voxels between them: rays change between
+    samples that read zero, which go on asking the mask, and ones that do not."""
+    hh, torch = gpu
+    dims = (41, 36, 33)
+    g = np.random.default_rng(gap)
+    z, y, x = hi.voxel_centres(dims)
+    r = np.sqrt((x - 20.0) ** 2 + (y - 18.0) ** 2 + (z - 16.0) ** 2)
+    dn = np.where(r % (2 * gap + 2) < gap + 2, -3e-5 * (1 + 0.2 * g.random(r.shape)), 0.0)
+    dn = dn.astype(np.float32)
+    bg = hi.checker_background()
+    bg_t = torch.from_numpy(bg).cuda()
+    vol = hh.hh_volume_from_dn(torch.from_numpy(dn.ravel()).cuda(), hh.make_grid(dims, 1.0, storage))
+    vol4 = export_volume(hh, torch, vol, dims)
+    cams = f32([hi.orbit_camera(dims, 25.0, 15.0, 37, 23), hi.orbit_camera(dims, 160.0, -40.0, 21, 29)])
+    adaptive = f32(hi.params_euler_adaptive(dims, theta_max=3e-3))
+    fixed = f32(hi.params_rk4_fixed(dims, 0.5))
+    fixed["stepper"] = "euler"
+    for params in (adaptive, fixed):
+        for cam, g in zip(cams, gpu_trace(hh, torch, vol, cams, params, bg_t)):
+            ref = oracle_lib.trace_grid(vol4, cam, params, bg)
+            assert_parity_conditioned(g, ref, oracle_lib, {"kind": "grid", "vol4": vol4}, dims, cam,
+                                      params)
+    vol.close()
+
+
 def test_volume_beyond_4_gib(gpu):
     """dn = c x in the far half of a grid whose FP32 volume exceeds 4 GiB, rays
     along -z from the far corner, all their samples beyond the 4 GiB: the
