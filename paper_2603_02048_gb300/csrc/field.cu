@@ -74,7 +74,7 @@ __device__ __forceinline__ uint2 pack16(const Voxel& v, float rs_n, float rs_g) 
 // by the voxel itself and the factor 1 instead of 1/2. Threads of the padding
 // compute a clamped voxel, which does not change a maximum and is not stored.
 // What bounds it: DRAM and its latency. 256^3 FP32: 58 us for the 285 MB it
-// moves (74 with a thread per column and 16-byte stores), FP16: maxima 33, store
+// moves (74 with a thread per column and 16-byte stores), FP16: maxima 31, store
 // 46 us (38 and 66). 5 resident blocks (48 registers) against 4 take 4 % off a
 // 512^3 FP16 build.
 constexpr int field_blocks(int mode) { return mode == 1 ? 4 : 5; }

@@ -45,7 +45,7 @@
 // 32 views of a 512^3 FP16 volume: 86 % of the pipe. RK4 with few rays is bound
 // by the four serial samples a step, ~340 cycles each. Against 2x2x2 bricks,
 // scalar state and IEEE approximations the step took these launches from 360 to
-// 285, 1227 to 1035 us and 10.1 to 9.15 ms.
+// 277, 1227 to 1035 us and 10.1 to 8.84 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
