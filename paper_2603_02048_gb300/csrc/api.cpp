@@ -101,16 +101,6 @@ namespace {
 
 cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 
-// Largest grid the kernels index with 32-bit per-axis coordinates and
-// 64-bit linear offsets.
-constexpr int kMaxAxis = 1 << 14;
-
-// Voxels of the grid with its one-voxel halo, every axis padded to even. A
-// ZPAIR volume pads its rows further, which adds at most three quarters.
-size_t stored_voxels(const hh_grid* g) {
-    return static_cast<size_t>((g->nx + 3) / 2) * ((g->ny + 3) / 2) * ((g->nz + 3) / 2) * 8;
-}
-
 hh_status check_grid(const hh_grid* g, bool need_h) {
     if (!g) return fail(HH_ERR_INVALID_ARG, "grid is NULL");
     if (g->nx < 2 || g->ny < 2 || g->nz < 2 || g->nx > kMaxAxis || g->ny > kMaxAxis ||
@@ -119,7 +109,7 @@ hh_status check_grid(const hh_grid* g, bool need_h) {
                     g->ny, g->nz, kMaxAxis);
     if (g->storage != HH_STORE_FP32 && g->storage != HH_STORE_FP16_SCALED)
         return fail(HH_ERR_INVALID_ARG, "unknown storage %d", g->storage);
-    if (stored_voxels(g) > (size_t(1) << 31))
+    if (stored_voxels(g->nx, g->ny, g->nz) > kMaxStored)
         return fail(HH_ERR_INVALID_ARG, "grid %d x %d x %d: more than 2^31 stored voxels", g->nx,
                     g->ny, g->nz);
     if (need_h && !(g->h_kernel > 0.0f && std::isfinite(g->h_kernel)))
@@ -150,15 +140,15 @@ hh_status new_volume(const hh_grid* g, hh_volume* out) {
     v->storage = g->storage;
     v->h_kernel = g->h_kernel;
     v->layout = HH_LAYOUT_ZPAIR;
-    v->row = zpair_row(g->nx, g->storage);
+    const unsigned voxel_bytes = g->storage == HH_STORE_FP32 ? 16 : 8;
+    v->row = zpair_row(g->nx, voxel_bytes);
     v->pair = zpair_pair(v->row, g->ny);
-    const size_t voxel_bytes = g->storage == HH_STORE_FP32 ? 16 : 8;
-    v->bytes = stored_voxels(g) * voxel_bytes;
+    v->bytes = stored_voxels(g->nx, g->ny, g->nz) * voxel_bytes;
     // the free-corner mask, its build scratch (a bit per element and voxel)
     // and the sparse flag follow the data in the same allocation; all of it
     // starts zero: no element is marked free before the first build
     const size_t pairs = (static_cast<size_t>(g->nz) + 3) / 2;
-    const size_t elements = static_cast<size_t>(v->pair) * pairs;
+    const size_t elements = zpair_elements(v->pair, g->nz);
     const size_t mask_words = (elements + 31) / 32;
     // (the mask kernel reads up to a slice, two rows and a word past the last)
     v->nz_words = (static_cast<unsigned>(g->nx) + 31u) / 32u;

@@ -8,6 +8,7 @@
 #include <cstdint>
 
 #include "hh.h"
+#include "zpair.h"
 
 // FP16 storage scales a channel group by the smallest power of two that maps
 // its largest |value| to at most this code (so to more than half of it), and
@@ -37,17 +38,8 @@
 //          16), and row = 6 (mod 8) on FP32 storage (1080p view of a dense 256^3
 //          volume 365 us; 376 at 12 (mod 16), 470 at 8), 12 (mod 16) on FP16 (32
 //          views of a 512^3 volume 9.13 ms against 9.15 to 9.60).
+// zpair.h has the strides and the corner addresses.
 enum { HH_LAYOUT_LINEAR = 0, HH_LAYOUT_ZPAIR = 1 };
-
-// ZPAIR strides in elements: of a row, and of a pair of slices. (A grid within
-// the size limit of the entry points has less than 2^32 elements.)
-inline unsigned zpair_row(int nx, int storage) {
-    const unsigned n = 2u * (static_cast<unsigned>(nx) + 2u);
-    return storage == HH_STORE_FP32 ? (n + 1u) / 8u * 8u + 6u : (n + 3u) / 16u * 16u + 12u;
-}
-inline unsigned zpair_pair(unsigned row, int ny) {
-    return (row * (static_cast<unsigned>(ny) + 2u) + 13u) / 16u * 16u + 2u;
-}
 
 struct hh_volume_s {
     int nx, ny, nz;
@@ -223,7 +215,7 @@ struct ServeWorkerArgs {
 // Resident blocks per SM of the worker for a launch shape, and its launch
 // (VolArgs from `like`: dims, storage, schedule, background; the volume data
 // and scales come from each job).
-int serve_worker_blocks_per_sm(int storage, int stepper, int adaptive, int threads);
+int serve_worker_blocks_per_sm(const hh_volume_s* like, const hh_step_params& P, int threads);
 cudaError_t launch_serve_worker(const hh_volume_s* like, const hh_step_params& P,
                                 const hh_background& bg, const ServeWorkerArgs& W, int blocks,
                                 int threads, cudaStream_t s);

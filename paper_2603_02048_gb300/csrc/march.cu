@@ -89,8 +89,7 @@ struct VolArgs {
     const float* scales;
     const unsigned* sparse;  // whether the volume's free-corner mask is worth testing
     int nx, ny, nz;
-    unsigned row, half_pair;      // ZPAIR strides of a row, and half of a pair of slices (elements)
-    unsigned row_bytes, up_bytes; // a row, and the step from an odd slice to the next - 1 element
+    ZPairStrides strides;
     unsigned long long mask_off;  // bytes from a volume's data to its free-corner mask
     float bias;         // power of two above every coordinate and step
     float bias_u;       // bias - 1/2: (hi - bias_u) + lo is the lattice coordinate
@@ -287,12 +286,8 @@ __device__ __forceinline__ float4 xlerp_fp16(uint2 a, uint2 b, float2 tt) {
 __device__ unsigned long long g_bounds_violations;
 #endif
 
-// How a kernel addresses the volume. ADDR_BASE: at V.vol, below 4 GiB, as
-// 32-bit byte offsets from base addresses the whole grid shares, which cost a
-// load no address arithmetic (FP16 384^3 4K view: 1733 against 1657 us).
-// ADDR_ANY: at a pointer of the caller's (the serving worker's jobs) or of any
-// size, with 64-bit addresses.
-enum { ADDR_BASE = 0, ADDR_ANY = 1 };
+// The volume a kernel samples: with ADDR_BASE (zpair.h) the one at V.vol, else the
+// one at the pointer passed.
 
 // Returns false, leaving s unset, for a sample whose eight corners are all
 // zero (the zero sample), read off the free-corner mask if `ask`. MASK = false
@@ -320,12 +315,8 @@ __device__ __forceinline__ bool fetch_nonzero(const VolArgs& A, const void* __re
 #else
     (void)flags;
 #endif
-    // ZPAIR element of corner (ix, iy, iz): (iz >> 1) pair + iy row + 2 ix + (iz
-    // & 1), the pair's half taken out by the parity
     const unsigned odd = static_cast<unsigned>(iz) & 1u;
-    const unsigned b = static_cast<unsigned>(iz) * A.half_pair +
-                       static_cast<unsigned>(iy) * A.row + 2u * static_cast<unsigned>(ix) -
-                       odd * (A.half_pair - 1u);
+    const unsigned b = zpair_element(A.strides, ix, iy, iz, odd);
     // the zero sample's bit: b & 31 of word b >> 5 (the funnel shift takes the
     // shift count mod 32)
     const char* base = static_cast<const char*>(ADDR == ADDR_BASE ? A.vol : vol);
@@ -333,25 +324,9 @@ __device__ __forceinline__ bool fetch_nonzero(const VolArgs& A, const void* __re
         const unsigned w = __ldg(reinterpret_cast<const unsigned*>(base + A.mask_off) + (b >> 5));
         if (__funnelshift_r(w, w, b) & 1u) return false;
     }
-    // The other corners: the next column is 2 elements on, the next row `row`,
-    // the next slice 1 for an even slice, else pair - 1.
     using V = typename std::conditional<STORAGE == HH_STORE_FP32, float4, uint2>::type;
-    constexpr unsigned size = sizeof(V);
-    const unsigned up = odd * A.up_bytes + size;
     const V *c00, *c10, *c01, *c11;  // corners (ix, iy + 0 or 1, iz + 0 or 1)
-    if (ADDR == ADDR_BASE) {
-        const char* next = base + A.row_bytes;
-        const unsigned at = b * size, above = at + up;
-        c00 = reinterpret_cast<const V*>(base + at);
-        c10 = reinterpret_cast<const V*>(next + at);
-        c01 = reinterpret_cast<const V*>(base + above);
-        c11 = reinterpret_cast<const V*>(next + above);
-    } else {
-        c00 = reinterpret_cast<const V*>(base) + b;
-        c01 = reinterpret_cast<const V*>(reinterpret_cast<const char*>(c00) + up);
-        c10 = reinterpret_cast<const V*>(reinterpret_cast<const char*>(c00) + A.row_bytes);
-        c11 = reinterpret_cast<const V*>(reinterpret_cast<const char*>(c01) + A.row_bytes);
-    }
+    zpair_corners<ADDR>(A.strides, base, b, odd, c00, c10, c01, c11);
     float4 c;
     if constexpr (STORAGE == HH_STORE_FP16_SCALED) {
         // lerps along x (the second corner converted inside the subtraction),
@@ -1099,7 +1074,7 @@ constexpr int worker_blocks(int storage, int stepper) {
     return batch_blocks(storage, stepper, false);
 }
 
-template <int STORAGE, int STEPPER, bool ADAPTIVE>
+template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
 __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
     serve_worker_kernel(const VolArgs V, const ServeWorkerArgs W) {
     extern __shared__ __align__(16) unsigned char s_raw[];  // a WorkerWarp per warp
@@ -1242,9 +1217,9 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
         const int px = (tx << tile_w_log2) + lx, py = ty * tile_h + ly;
         if (px < C.W && py < C.H) {
             RayState R;
-                    ray_begin<ADAPTIVE>(V, reinterpret_cast<const float*>(S.scales), C, px, py, R);
+            ray_begin<ADAPTIVE>(V, reinterpret_cast<const float*>(S.scales), C, px, py, R);
             if (R.flags & HH_FLAG_HIT)
-                ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>(
+                ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(
                     V, reinterpret_cast<const void*>(S.vol), S.sparse, R);
             ray_end(V, C, px, py, R);
         }
@@ -1270,9 +1245,9 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
     }
 }
 
-// ADDR_BASE wherever the volume's byte offsets fit 32 bits (V.mask_off is the
-// end of its data).
-bool addr_any(const VolArgs& V) { return V.mask_off >= (1ull << 32); }
+// Whether the volume needs ADDR_ANY: its byte offsets do not fit 32 bits (mask_off
+// is the end of its data).
+bool addr_any(unsigned long long mask_off) { return mask_off >= (1ull << 32); }
 
 template <int STORAGE, int STEPPER, bool ADAPTIVE>
 void launch_one(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
@@ -1286,7 +1261,7 @@ void launch_one(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
     float row = 0.5f * C.H;
     if (ahead > 0.0f) row = (C.b0 - up / ahead) / C.s;
     const int mid = static_cast<int>(fminf(fmaxf(row, 0.0f), C.H - 1.0f)) / 8;
-    if (addr_any(V))
+    if (addr_any(V.mask_off))
         launch_next(march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>, grid, block, s, V, C, mid);
     else
         launch_next(march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_BASE>, grid, block, s, V, C, mid);
@@ -1330,25 +1305,31 @@ struct BatchLaunch {
                     int tile_w, unsigned* counter, int refill_min, const uint2* order, int group,
                     int blocks, int threads, cudaStream_t s) {
         const size_t smem = (n_views + 1) * sizeof(int);
-        batch_kernel<ST, SP, AD>(addr_any(V), refill_min)<<<blocks, threads, smem, s>>>(
+        batch_kernel<ST, SP, AD>(addr_any(V.mask_off), refill_min)<<<blocks, threads, smem, s>>>(
             V, views, n_views, total_tiles, tile_w, counter, refill_min, order,
             refill_min >= 32 ? group : 0);
     }
 };
+
+// The worker on volumes of one grid and storage: all below 4 GiB, or none.
+template <int ST, int SP, bool AD>
+auto worker_kernel(bool any) {
+    return any ? serve_worker_kernel<ST, SP, AD, ADDR_ANY> : serve_worker_kernel<ST, SP, AD, ADDR_PTR>;
+}
 
 template <int ST, int SP, bool AD>
 struct WorkerLaunch {
     static void run(const VolArgs& V, const ServeWorkerArgs& W, int blocks, int threads,
                     cudaStream_t s) {
         const size_t smem = (threads / 32) * sizeof(WorkerWarp);
-        serve_worker_kernel<ST, SP, AD><<<blocks, threads, smem, s>>>(V, W);
+        worker_kernel<ST, SP, AD>(addr_any(V.mask_off))<<<blocks, threads, smem, s>>>(V, W);
     }
 };
 
 template <int ST, int SP, bool AD>
 struct WorkerOccupancy {
-    static void run(int threads, int* blocks_per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, serve_worker_kernel<ST, SP, AD>,
+    static void run(bool any, int threads, int* blocks_per_sm) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, worker_kernel<ST, SP, AD>(any),
                                                       threads, (threads / 32) * sizeof(WorkerWarp));
     }
 };
@@ -1369,11 +1350,7 @@ VolArgs make_vol_args(const hh_volume_s* vol, const hh_step_params& P, const hh_
     A.ny = vol->ny;
     A.nz = vol->nz;
     A.sparse = vol->sparse_dev;
-    A.row = vol->row;
-    A.half_pair = vol->pair / 2;
-    const unsigned voxel_bytes = vol->storage == HH_STORE_FP32 ? 16u : 8u;
-    A.row_bytes = vol->row * voxel_bytes;
-    A.up_bytes = (vol->pair - 2u) * voxel_bytes;
+    A.strides = zpair_strides(vol->row, vol->pair, vol->storage == HH_STORE_FP32 ? 16u : 8u);
     A.mask_off = vol->mask_off;
     // bias: a power of two B with B >= 2 * step and B >= extent + step + 1, so
     // positions in [-step, extent + step] keep hi in [B/2, 2B - 1] and both
@@ -1474,9 +1451,10 @@ int build_view_table(const hh_camera* cams, const hh_view_out* outs, int n, int 
     return static_cast<int>(tiles);
 }
 
-int serve_worker_blocks_per_sm(int storage, int stepper, int adaptive, int threads) {
+int serve_worker_blocks_per_sm(const hh_volume_s* like, const hh_step_params& P, int threads) {
     int bps = 0;
-    dispatch<WorkerOccupancy>(storage, stepper, adaptive, threads, &bps);
+    dispatch<WorkerOccupancy>(like->storage, P.stepper, P.adaptive, addr_any(like->mask_off), threads,
+                              &bps);
     return max(bps, 1);
 }
 
@@ -1607,7 +1585,7 @@ int resident_blocks(hh_batch b, int threads, int refill_min) {
     int bps = 0;
     const size_t smem = (b->cams.size() + 1) * sizeof(int);
     hh::dispatch<hh::BatchOccupancy>(b->vol->storage, b->params.stepper, b->params.adaptive,
-                                     threads, smem, b->vol->mask_off >= (1ull << 32), refill_min, &bps);
+                                     threads, smem, hh::addr_any(b->vol->mask_off), refill_min, &bps);
     return std::max(bps, 1);
 }
 

@@ -361,8 +361,7 @@ void hh_server_s::launch_worker() {
     W.entry_ns = kEntryNs;
     const int bps = cfg.blocks_per_sm > 0
                         ? cfg.blocks_per_sm
-                        : hh::serve_worker_blocks_per_sm(cls_vol->storage, cls_params.stepper,
-                                                         cls_params.adaptive, cfg.block_threads);
+                        : hh::serve_worker_blocks_per_sm(cls_vol, cls_params, cfg.block_threads);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(work_stream, published, 0);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctl_dev + 3, 0, 3 * sizeof(int), work_stream);
     if (e == cudaSuccess)
