@@ -222,20 +222,42 @@ __device__ __forceinline__ float4 lerp4x2(float4 a, float4 b, float2 tt) {
     return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
-// Hardware approximate square root and division (PTX *.approx.ftz.f32, ~1 ulp):
-// without .ftz each carries instructions for subnormal operands (same march:
-// 330 against 320 us). A subnormal |g_perp|^2 taken as 0 moves
-// |g_perp| by less than 1.1e-19, which eps outweighs; the other operands are
-// subnormal only where the step length or eps itself is.
+// The step length of a kernel: a fixed one, Eq. 18's with the approximations
+// below that take subnormals for zero, or (LEN_SUBNORMAL, either of them) with
+// ones that do not. step_len() picks for a launch.
+enum { LEN_FIXED = 0, LEN_EQ18 = 1, LEN_SUBNORMAL = 2 };
+
+// Hardware approximate square root and division (PTX *.approx[.ftz].f32, ~1 ulp):
+// without .ftz each carries instructions for subnormal operands (march of the
+// 1080p frame: 330 against 320 us).
+template <int LEN>
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    if (LEN == LEN_SUBNORMAL)
+        asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    else
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+template <int LEN>
 __device__ __forceinline__ float div_approx(float a, float b) {
     float r;
-    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    if (LEN == LEN_SUBNORMAL)
+        asm("div.approx.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    else
+        asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
+}
+
+// What .ftz drops does not show where a subnormal |g_perp|^2, |g_perp| below
+// 1.1e-19, is at most 2^-24 of eps, and the tolerance and the steps themselves are
+// far from subnormal (n, near 1, takes them no further). Other parameters, which
+// no scene in use has, march with LEN_SUBNORMAL.
+int step_len(const hh_step_params& P) {
+    const float least = 0x1p-100f;
+    if (!P.adaptive) return P.h_fixed < least ? LEN_SUBNORMAL : LEN_FIXED;
+    const bool tiny = P.eps < 0x1p-39f || P.h_min < least || (P.theta_max > 0.0f && P.theta_max < least);
+    return tiny ? LEN_SUBNORMAL : LEN_EQ18;
 }
 
 // Lattice cell and weight along one axis from the lattice coordinate u =
@@ -384,11 +406,12 @@ __device__ __forceinline__ Sample fetch(const VolArgs& A, const void* __restrict
     return s;
 }
 
-// Eq. 18 (second form) or the fixed step.
-template <bool ADAPTIVE>
+// Eq. 18 (second form) or the fixed step (LEN_SUBNORMAL's is Eq. 18's with h_min =
+// h_max).
+template <int LEN>
 __device__ __forceinline__ float step_length(const VolArgs& A, float n, float gperp_norm) {
-    if (!ADAPTIVE) return A.h_fixed;
-    return fminf(fmaxf(div_approx(n * A.theta, gperp_norm + A.eps), A.h_min), A.h_max);
+    if (LEN == LEN_FIXED) return A.h_fixed;
+    return fminf(fmaxf(div_approx<LEN>(n * A.theta, gperp_norm + A.eps), A.h_min), A.h_max);
 }
 
 // Eq. 16's normalize, in deflection form: returns d' with w_ref + d' the unit
@@ -582,22 +605,22 @@ __device__ __forceinline__ float exit_fraction(const VolArgs& A, float3 hi, floa
 // and s_g are powers of two, so every such product is exact and the results
 // equal those of scaling the sample first: n = 1 + dn s_n is one rounding
 // either way, and |g_perp| = s_g |g_perp / s_g| exactly.
-template <int STORAGE>
+template <int STORAGE, int LEN>
 __device__ __forceinline__ float3 perp_of(const Sample& s, float3 w, float s_n, float s_g,
                                           float& n, float& gperp_norm) {
     n = STORAGE == HH_STORE_FP32 ? 1.0f + s.dn : fmaf(s.dn, s_n, 1.0f);
     const float3 g = make_float3(s.gx, s.gy, s.gz);
     const float3 gp = fma_p(-dot(w, g), w, g);
-    gperp_norm = sqrt_approx(dot(gp, gp));
+    gperp_norm = sqrt_approx<LEN>(dot(gp, gp));
     if (STORAGE != HH_STORE_FP32) gperp_norm *= s_g;
     return gp;
 }
-template <int STORAGE, int ADDR, bool MASK, bool CLAMP>
+template <int STORAGE, int LEN, int ADDR, bool MASK, bool CLAMP>
 __device__ __forceinline__ float3 perp_rate(const VolArgs& A, const void* __restrict__ vol,
                                             float3 u, float3 w, float s_n, float s_g, float& n,
                                             float& gperp_norm, uint32_t& flags) {
-    return perp_of<STORAGE>(fetch<STORAGE, ADDR, MASK, CLAMP>(A, vol, u, flags), w, s_n, s_g, n,
-                            gperp_norm);
+    return perp_of<STORAGE, LEN>(fetch<STORAGE, ADDR, MASK, CLAMP>(A, vol, u, flags), w, s_n, s_g, n,
+                                 gperp_norm);
 }
 
 // Per-ray state of the march: primary direction w_ref, deflection d, biased
@@ -627,13 +650,13 @@ __device__ __forceinline__ void tile_pixel(int p, int tile_w_log2, int& x, int& 
 }
 
 // Ray generation and slab entry (flags = HIT when the ray enters the box).
-template <bool ADAPTIVE>
+template <int LEN>
 __device__ __forceinline__ void ray_begin(const VolArgs& V, const float* __restrict__ scales,
                                           const ViewArgs& C, int px, int py, RayState& R) {
     R.wr = primary_ray(C, px, py);
     R.sn = __ldg(scales);
     R.sg = __ldg(scales + 1);
-    R.ds0 = step_length<ADAPTIVE>(V, 1.0f, 0.0f);
+    R.ds0 = step_length<LEN>(V, 1.0f, 0.0f);
     R.last = 0.0f;
     R.k = 0;
     R.flags = 0;
@@ -661,7 +684,7 @@ __device__ __forceinline__ void ray_begin(const VolArgs& V, const float* __restr
 // Returns true when the step leaves the box: then R.hi and R.d, of no further
 // use to the march, hold the exit point on the face and the new direction (six
 // registers that the loop need not carry).
-template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR, bool MASK>
+template <int STORAGE, int STEPPER, int LEN, int ADDR, bool MASK>
 __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restrict__ vol,
                                          RayState& R) {
     const float B = V.bias;
@@ -673,25 +696,25 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
     if (STEPPER == HH_STEP_RK4) {
         float n1, gpn, n2, n3, n4, unused;
         const float3 w1 = wr + d;
-        const float3 gp1 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, C, w1, R.sn, R.sg, n1, gpn, R.flags);
-        ds = step_length<ADAPTIVE>(V, n1, gpn);
+        const float3 gp1 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, C, w1, R.sn, R.sg, n1, gpn, R.flags);
+        ds = step_length<LEN>(V, n1, gpn);
         const float hds = 0.5f * ds;
-        const float3 k1 = (div_approx(1.0f, n1) * gsc) * gp1;
+        const float3 k1 = (div_approx<LEN>(1.0f, n1) * gsc) * gp1;
         const float3 d2 = fma3(hds, k1, d);
         const float3 w2 = wr + d2;
-        const float3 gp2 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(hds, w1, C), w2, R.sn, R.sg, n2,
+        const float3 gp2 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, fma3(hds, w1, C), w2, R.sn, R.sg, n2,
                                                     unused, R.flags);
-        const float3 k2 = (div_approx(1.0f, n2) * gsc) * gp2;
+        const float3 k2 = (div_approx<LEN>(1.0f, n2) * gsc) * gp2;
         const float3 d3 = fma3(hds, k2, d);
         const float3 w3 = wr + d3;
-        const float3 gp3 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(hds, w2, C), w3, R.sn, R.sg, n3,
+        const float3 gp3 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, fma3(hds, w2, C), w3, R.sn, R.sg, n3,
                                                     unused, R.flags);
-        const float3 k3 = (div_approx(1.0f, n3) * gsc) * gp3;
+        const float3 k3 = (div_approx<LEN>(1.0f, n3) * gsc) * gp3;
         const float3 d4 = fma3(ds, k3, d);
         const float3 w4 = wr + d4;
-        const float3 gp4 = perp_rate<STORAGE, ADDR, MASK, true>(V, vol, fma3(ds, w3, C), w4, R.sn, R.sg, n4,
+        const float3 gp4 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, fma3(ds, w3, C), w4, R.sn, R.sg, n4,
                                                     unused, R.flags);
-        const float3 k4 = (div_approx(1.0f, n4) * gsc) * gp4;
+        const float3 k4 = (div_approx<LEN>(1.0f, n4) * gsc) * gp4;
         // k1 + 2 (k2 + k3) + k4 (every k is a product: the adds are kept
         // unfused, __fadd_rn, so no product is folded into them)
         const float3 ksum =
@@ -716,9 +739,9 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
         if (fetch_nonzero<STORAGE, ADDR, MASK, false>(V, vol, C, R.last == 0.0f, R.flags, smp)) {
             if (MASK) R.last = smp.dn;
             float n, gpn;
-            const float3 gp = perp_of<STORAGE>(smp, add_p(wr, d), R.sn, R.sg, n, gpn);
-            ds = step_length<ADAPTIVE>(V, n, gpn);
-            d1 = fma_p(div_approx(ds, n) * gsc, gp, d);
+            const float3 gp = perp_of<STORAGE, LEN>(smp, add_p(wr, d), R.sn, R.sg, n, gpn);
+            ds = step_length<LEN>(V, n, gpn);
+            d1 = fma_p(div_approx<LEN>(ds, n) * gsc, gp, d);
         } else {
             // the zero sample: n = 1 and g_perp = 0 exactly, so the branch
             // above would give the step length ds0 (the same operations on
@@ -764,16 +787,16 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
 // Marches a ray that entered the box until it leaves it or runs out of steps.
 // `sparse` (the same for every ray of the volume) picks the loop that tests the
 // free-corner mask or the one that does not.
-template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
+template <int STORAGE, int STEPPER, int LEN, int ADDR>
 __device__ __forceinline__ void ray_march(const VolArgs& V, const void* __restrict__ vol,
                                           unsigned sparse, RayState& R) {
     if (sparse) {
         while (R.k < V.max_steps &&
-               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, vol, R)) {
+               !ray_step<STORAGE, STEPPER, LEN, ADDR, true>(V, vol, R)) {
         }
     } else {
         while (R.k < V.max_steps &&
-               !ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, vol, R)) {
+               !ray_step<STORAGE, STEPPER, LEN, ADDR, false>(V, vol, R)) {
         }
     }
 }
@@ -840,7 +863,7 @@ __device__ __forceinline__ int row_from(int i, int n, int mid) {
 // the 256^3 plume 295 against 285). Its blocks never release_next(): those of
 // another view behind it would gather on the SMs that empty first (the RK4 view,
 // launches back to back: 87.5 us, without 62.1, launched as ordinary ones 64.6).
-template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
+template <int STORAGE, int STEPPER, int LEN, int ADDR>
 __global__ void __launch_bounds__(128, march_blocks(STORAGE, STEPPER))
     march_kernel(const VolArgs V, const ViewArgs C, const int mid) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -852,9 +875,9 @@ __global__ void __launch_bounds__(128, march_blocks(STORAGE, STEPPER))
     const int py = row_from(blockIdx.y, gridDim.y, mid) * 8 + (warp >> 1) * 4 + ty;
     if (px >= C.W || py >= C.H) return;
     RayState R;
-    ray_begin<ADAPTIVE>(V, after_wait(V.scales), C, px, py, R);
+    ray_begin<LEN>(V, after_wait(V.scales), C, px, py, R);
     if (R.flags & HH_FLAG_HIT)
-        ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, __ldg(after_wait(V.sparse)), R);
+        ray_march<STORAGE, STEPPER, LEN, ADDR>(V, V.vol, __ldg(after_wait(V.sparse)), R);
     ray_end(V, C, px, py, R);
 }
 
@@ -899,7 +922,7 @@ __device__ __forceinline__ void tile_of(int t, int n_views, const int* s_begin,
 // march them side by side on one SM, sharing its L1, and meet at a barrier
 // before the next group, as march_kernel's blocks do when they retire. The
 // per-ray arithmetic is march_kernel's.
-template <int STORAGE, int STEPPER, bool ADAPTIVE, bool REFILL, int ADDR>
+template <int STORAGE, int STEPPER, int LEN, bool REFILL, int ADDR>
 __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
     march_batch_kernel(const VolArgs V, const ViewArgs* __restrict__ views, int n_views,
                        int total_tiles, int tile_w, unsigned* __restrict__ counter,
@@ -952,9 +975,9 @@ __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
             const int px = (tx << tile_w_log2) + lx, py = ty * (32 >> tile_w_log2) + ly;
             if (px < C.W && py < C.H) {
                 RayState R;
-                ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
+                ray_begin<LEN>(V, V.scales, C, px, py, R);
                 if (R.flags & HH_FLAG_HIT)
-                    ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(V, V.vol, sparse, R);
+                    ray_march<STORAGE, STEPPER, LEN, ADDR>(V, V.vol, sparse, R);
                 ray_end(V, C, px, py, R);
             }
         }
@@ -991,7 +1014,7 @@ __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
                     py = tile_y * (32 >> tile_w_log2) + ly;
                     vi = tile_view;
                     if (px < C.W && py < C.H) {
-                        ray_begin<ADAPTIVE>(V, V.scales, C, px, py, R);
+                        ray_begin<LEN>(V, V.scales, C, px, py, R);
                         if ((R.flags & HH_FLAG_HIT) && V.max_steps > 0) have = true;
                         else ray_end(V, C, px, py, R);
                     }
@@ -1006,8 +1029,8 @@ __global__ void __launch_bounds__(256, batch_blocks(STORAGE, STEPPER, REFILL))
         }
         if (have) {
             const bool left =
-                sparse ? ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, true>(V, V.vol, R)
-                       : ray_step<STORAGE, STEPPER, ADAPTIVE, ADDR, false>(V, V.vol, R);
+                sparse ? ray_step<STORAGE, STEPPER, LEN, ADDR, true>(V, V.vol, R)
+                       : ray_step<STORAGE, STEPPER, LEN, ADDR, false>(V, V.vol, R);
             if (left || R.k >= V.max_steps) {
                 ray_end(V, views[vi], px, py, R);
                 have = false;
@@ -1074,7 +1097,7 @@ constexpr int worker_blocks(int storage, int stepper) {
     return batch_blocks(storage, stepper, false);
 }
 
-template <int STORAGE, int STEPPER, bool ADAPTIVE, int ADDR>
+template <int STORAGE, int STEPPER, int LEN, int ADDR>
 __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
     serve_worker_kernel(const VolArgs V, const ServeWorkerArgs W) {
     extern __shared__ __align__(16) unsigned char s_raw[];  // a WorkerWarp per warp
@@ -1217,9 +1240,9 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
         const int px = (tx << tile_w_log2) + lx, py = ty * tile_h + ly;
         if (px < C.W && py < C.H) {
             RayState R;
-            ray_begin<ADAPTIVE>(V, reinterpret_cast<const float*>(S.scales), C, px, py, R);
+            ray_begin<LEN>(V, reinterpret_cast<const float*>(S.scales), C, px, py, R);
             if (R.flags & HH_FLAG_HIT)
-                ray_march<STORAGE, STEPPER, ADAPTIVE, ADDR>(
+                ray_march<STORAGE, STEPPER, LEN, ADDR>(
                     V, reinterpret_cast<const void*>(S.vol), S.sparse, R);
             ray_end(V, C, px, py, R);
         }
@@ -1248,8 +1271,11 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
 // Whether the volume needs ADDR_ANY: its byte offsets do not fit 32 bits (mask_off
 // is the end of its data).
 bool addr_any(unsigned long long mask_off) { return mask_off >= (1ull << 32); }
+// The form of a kernel for volumes that do not: `addr`, or ADDR_ANY, compiled
+// anyway, where speed does not matter.
+constexpr int narrow(int len, int addr) { return len == LEN_SUBNORMAL ? ADDR_ANY : addr; }
 
-template <int STORAGE, int STEPPER, bool ADAPTIVE>
+template <int STORAGE, int STEPPER, int LEN>
 void launch_one(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
     const dim3 block(128);
     const dim3 grid((C.W + 15) / 16, (C.H + 7) / 8);
@@ -1262,83 +1288,88 @@ void launch_one(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
     if (ahead > 0.0f) row = (C.b0 - up / ahead) / C.s;
     const int mid = static_cast<int>(fminf(fmaxf(row, 0.0f), C.H - 1.0f)) / 8;
     if (addr_any(V.mask_off))
-        launch_next(march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_ANY>, grid, block, s, V, C, mid);
+        launch_next(march_kernel<STORAGE, STEPPER, LEN, ADDR_ANY>, grid, block, s, V, C, mid);
     else
-        launch_next(march_kernel<STORAGE, STEPPER, ADAPTIVE, ADDR_BASE>, grid, block, s, V, C, mid);
+        launch_next(march_kernel<STORAGE, STEPPER, LEN, narrow(LEN, ADDR_BASE)>, grid, block,
+                    s, V, C, mid);
 }
 
-// Calls F<STORAGE, STEPPER, ADAPTIVE>::run(args...) for the runtime choice.
-template <template <int, int, bool> class F, typename... Args>
-void dispatch(int storage, int stepper, int adaptive, Args&&... args) {
-    const bool fp16 = storage == HH_STORE_FP16_SCALED, rk4 = stepper == HH_STEP_RK4;
-    if (!fp16 && !rk4 && !adaptive) F<HH_STORE_FP32, HH_STEP_EULER_PAPER, false>::run(args...);
-    if (!fp16 && !rk4 && adaptive) F<HH_STORE_FP32, HH_STEP_EULER_PAPER, true>::run(args...);
-    if (!fp16 && rk4 && !adaptive) F<HH_STORE_FP32, HH_STEP_RK4, false>::run(args...);
-    if (!fp16 && rk4 && adaptive) F<HH_STORE_FP32, HH_STEP_RK4, true>::run(args...);
-    if (fp16 && !rk4 && !adaptive) F<HH_STORE_FP16_SCALED, HH_STEP_EULER_PAPER, false>::run(args...);
-    if (fp16 && !rk4 && adaptive) F<HH_STORE_FP16_SCALED, HH_STEP_EULER_PAPER, true>::run(args...);
-    if (fp16 && rk4 && !adaptive) F<HH_STORE_FP16_SCALED, HH_STEP_RK4, false>::run(args...);
-    if (fp16 && rk4 && adaptive) F<HH_STORE_FP16_SCALED, HH_STEP_RK4, true>::run(args...);
+// Calls F<STORAGE, STEPPER, LEN>::run(args...) for the runtime choice.
+template <template <int, int, int> class F, int STORAGE, int STEPPER, typename... Args>
+void dispatch_len(int len, Args&&... args) {
+    if (len == LEN_FIXED) F<STORAGE, STEPPER, LEN_FIXED>::run(args...);
+    else if (len == LEN_EQ18) F<STORAGE, STEPPER, LEN_EQ18>::run(args...);
+    else F<STORAGE, STEPPER, LEN_SUBNORMAL>::run(args...);
+}
+template <template <int, int, int> class F, typename... Args>
+void dispatch(int storage, const hh_step_params& P, Args&&... args) {
+    const bool fp16 = storage == HH_STORE_FP16_SCALED, rk4 = P.stepper == HH_STEP_RK4;
+    const int len = step_len(P);
+    if (!fp16 && !rk4) dispatch_len<F, HH_STORE_FP32, HH_STEP_EULER_PAPER>(len, args...);
+    else if (!fp16) dispatch_len<F, HH_STORE_FP32, HH_STEP_RK4>(len, args...);
+    else if (!rk4) dispatch_len<F, HH_STORE_FP16_SCALED, HH_STEP_EULER_PAPER>(len, args...);
+    else dispatch_len<F, HH_STORE_FP16_SCALED, HH_STEP_RK4>(len, args...);
 }
 
-template <int ST, int SP, bool AD>
+template <int ST, int SP, int LEN>
 struct SingleLaunch {
     static void run(const VolArgs& V, const ViewArgs& C, cudaStream_t s) {
-        launch_one<ST, SP, AD>(V, C, s);
+        launch_one<ST, SP, LEN>(V, C, s);
     }
 };
 
 // The batch kernel of a launch: refill_min >= 32 runs the tile-at-a-time
 // instantiation (REFILL = false).
-template <int ST, int SP, bool AD>
+template <int ST, int SP, int LEN>
 auto batch_kernel(bool any, int refill_min) {
     if (refill_min >= 32)
-        return any ? march_batch_kernel<ST, SP, AD, false, ADDR_ANY>
-                   : march_batch_kernel<ST, SP, AD, false, ADDR_BASE>;
-    return any ? march_batch_kernel<ST, SP, AD, true, ADDR_ANY>
-               : march_batch_kernel<ST, SP, AD, true, ADDR_BASE>;
+        return any ? march_batch_kernel<ST, SP, LEN, false, ADDR_ANY>
+                   : march_batch_kernel<ST, SP, LEN, false, narrow(LEN, ADDR_BASE)>;
+    return any ? march_batch_kernel<ST, SP, LEN, true, ADDR_ANY>
+               : march_batch_kernel<ST, SP, LEN, true, narrow(LEN, ADDR_BASE)>;
 }
 
-template <int ST, int SP, bool AD>
+template <int ST, int SP, int LEN>
 struct BatchLaunch {
     static void run(const VolArgs& V, const ViewArgs* views, int n_views, int total_tiles,
                     int tile_w, unsigned* counter, int refill_min, const uint2* order, int group,
                     int blocks, int threads, cudaStream_t s) {
         const size_t smem = (n_views + 1) * sizeof(int);
-        batch_kernel<ST, SP, AD>(addr_any(V.mask_off), refill_min)<<<blocks, threads, smem, s>>>(
+        batch_kernel<ST, SP, LEN>(addr_any(V.mask_off), refill_min)<<<blocks, threads, smem, s>>>(
             V, views, n_views, total_tiles, tile_w, counter, refill_min, order,
             refill_min >= 32 ? group : 0);
     }
 };
 
 // The worker on volumes of one grid and storage: all below 4 GiB, or none.
-template <int ST, int SP, bool AD>
+template <int ST, int SP, int LEN>
 auto worker_kernel(bool any) {
-    return any ? serve_worker_kernel<ST, SP, AD, ADDR_ANY> : serve_worker_kernel<ST, SP, AD, ADDR_PTR>;
+    return any ? serve_worker_kernel<ST, SP, LEN, ADDR_ANY>
+               : serve_worker_kernel<ST, SP, LEN, narrow(LEN, ADDR_PTR)>;
 }
 
-template <int ST, int SP, bool AD>
+template <int ST, int SP, int LEN>
 struct WorkerLaunch {
     static void run(const VolArgs& V, const ServeWorkerArgs& W, int blocks, int threads,
                     cudaStream_t s) {
         const size_t smem = (threads / 32) * sizeof(WorkerWarp);
-        worker_kernel<ST, SP, AD>(addr_any(V.mask_off))<<<blocks, threads, smem, s>>>(V, W);
+        worker_kernel<ST, SP, LEN>(addr_any(V.mask_off))<<<blocks, threads, smem, s>>>(V, W);
     }
 };
 
-template <int ST, int SP, bool AD>
+template <int ST, int SP, int LEN>
 struct WorkerOccupancy {
     static void run(bool any, int threads, int* blocks_per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, worker_kernel<ST, SP, AD>(any),
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, worker_kernel<ST, SP, LEN>(any),
                                                       threads, (threads / 32) * sizeof(WorkerWarp));
     }
 };
 
-template <int ST, int SP, bool AD>
+template <int ST, int SP, int LEN>
 struct BatchOccupancy {
     static void run(int threads, size_t smem, bool any, int refill_min, int* blocks_per_sm) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            blocks_per_sm, batch_kernel<ST, SP, AD>(any, refill_min), threads, smem);
+            blocks_per_sm, batch_kernel<ST, SP, LEN>(any, refill_min), threads, smem);
     }
 };
 
@@ -1366,10 +1397,10 @@ VolArgs make_vol_args(const hh_volume_s* vol, const hh_step_params& P, const hh_
     A.uy = static_cast<float>(vol->ny) + 0.5f;
     A.uz = static_cast<float>(vol->nz) + 0.5f;
     A.h_fixed = P.h_fixed;
-    A.h_min = P.h_min;
-    A.h_max = P.h_max;
-    A.theta = P.theta_max;
-    A.eps = P.eps;
+    A.h_min = P.adaptive ? P.h_min : P.h_fixed;
+    A.h_max = P.adaptive ? P.h_max : P.h_fixed;
+    A.theta = P.adaptive ? P.theta_max : 0.0f;
+    A.eps = P.adaptive ? P.eps : 1.0f;
     A.max_steps = P.max_steps;
     A.bg = bg.rgb8_dev;
     A.bgW = bg.width;
@@ -1426,7 +1457,7 @@ cudaError_t launch_trace(const hh_volume_s* vol, const hh_camera& cam, const hh_
     if (vol->layout != HH_LAYOUT_ZPAIR) return cudaErrorInvalidValue;
     const VolArgs V = make_vol_args(vol, P, bg);
     const ViewArgs C = make_view_args(cam, out, 8);
-    dispatch<SingleLaunch>(vol->storage, P.stepper, P.adaptive, V, C, s);
+    dispatch<SingleLaunch>(vol->storage, P, V, C, s);
     count_launch();
     return cudaGetLastError();
 }
@@ -1453,8 +1484,7 @@ int build_view_table(const hh_camera* cams, const hh_view_out* outs, int n, int 
 
 int serve_worker_blocks_per_sm(const hh_volume_s* like, const hh_step_params& P, int threads) {
     int bps = 0;
-    dispatch<WorkerOccupancy>(like->storage, P.stepper, P.adaptive, addr_any(like->mask_off), threads,
-                              &bps);
+    dispatch<WorkerOccupancy>(like->storage, P, addr_any(like->mask_off), threads, &bps);
     return max(bps, 1);
 }
 
@@ -1463,7 +1493,7 @@ cudaError_t launch_serve_worker(const hh_volume_s* like, const hh_step_params& P
                                 int threads, cudaStream_t s) {
     if (like->layout != HH_LAYOUT_ZPAIR) return cudaErrorInvalidValue;
     const VolArgs V = make_vol_args(like, P, bg);
-    dispatch<WorkerLaunch>(like->storage, P.stepper, P.adaptive, V, W, blocks, threads, s);
+    dispatch<WorkerLaunch>(like->storage, P, V, W, blocks, threads, s);
     count_launch();
     return cudaGetLastError();
 }
@@ -1584,8 +1614,8 @@ hh_status check_config(const hh_batch_config* c) {
 int resident_blocks(hh_batch b, int threads, int refill_min) {
     int bps = 0;
     const size_t smem = (b->cams.size() + 1) * sizeof(int);
-    hh::dispatch<hh::BatchOccupancy>(b->vol->storage, b->params.stepper, b->params.adaptive,
-                                     threads, smem, hh::addr_any(b->vol->mask_off), refill_min, &bps);
+    hh::dispatch<hh::BatchOccupancy>(b->vol->storage, b->params, threads, smem,
+                                     hh::addr_any(b->vol->mask_off), refill_min, &bps);
     return std::max(bps, 1);
 }
 
@@ -1603,8 +1633,8 @@ cudaError_t enqueue(hh_batch b, int blocks, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const int threads = b->cfg.block_threads;
     const hh::VolArgs V = hh::make_vol_args(b->vol, b->params, b->bg);
-    hh::dispatch<hh::BatchLaunch>(b->vol->storage, b->params.stepper, b->params.adaptive, V,
-                                  b->views_dev, static_cast<int>(b->cams.size()), b->total_tiles,
+    hh::dispatch<hh::BatchLaunch>(b->vol->storage, b->params, V, b->views_dev,
+                                  static_cast<int>(b->cams.size()), b->total_tiles,
                                   b->cfg.tile_w, b->counter_dev, b->cfg.refill_min,
                                   static_cast<const uint2*>(b->order_dev), b->cfg.tile_group,
                                   blocks, threads, s);
