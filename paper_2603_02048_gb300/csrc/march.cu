@@ -56,6 +56,7 @@
 #include <vector>
 
 #include "hh_internal.h"
+#include "texels.h"
 
 namespace hh {
 namespace {
@@ -431,27 +432,27 @@ __device__ __forceinline__ float3 renormalize(float3 w1, float3 d1) {
     return fma3(renorm_term(w1), w1, d1);
 }
 
-// Two neighbouring RGB8 texels, six bytes from p on, from the aligned 32-bit
-// words that hold them (no word without a byte of them is read): two loads, or
-// three where p is the last byte of a word, instead of six.
-__device__ __forceinline__ void texel_pair(const uint8_t* __restrict__ p, float2& r, float2& g,
-                                           float2& b) {
-    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
-    const unsigned* w = reinterpret_cast<const unsigned*>(at & ~uintptr_t(3));
-    const unsigned byte = static_cast<unsigned>(at) & 3u;
-    const unsigned w0 = __ldg(w), w1 = __ldg(w + 1), w2 = byte == 3u ? __ldg(w + 2) : 0u;
-    const unsigned lo = __funnelshift_r(w0, w1, 8u * byte), hi = __funnelshift_r(w1, w2, 8u * byte);
+struct LoadTexels {
+    __device__ __forceinline__ uint32_t operator()(const uint8_t* p) const { return __ldg(p); }
+    __device__ __forceinline__ uint32_t operator()(const uint32_t* p) const { return __ldg(p); }
+};
+
+// Channels of a pair of texels read as lo, hi.
+__device__ __forceinline__ void texel_channels(uint32_t lo, uint32_t hi, float2& r, float2& g,
+                                               float2& b) {
     r = make_float2(static_cast<float>(lo & 0xFFu), static_cast<float>(lo >> 24));
     g = make_float2(static_cast<float>((lo >> 8) & 0xFFu), static_cast<float>(hi & 0xFFu));
     b = make_float2(static_cast<float>((lo >> 16) & 0xFFu), static_cast<float>((hi >> 8) & 0xFFu));
 }
 
-// Bilinear colour of texel pairs p0 (row j) and p1 (row j + 1); value / 255.
-__device__ __forceinline__ float3 texel_lerp(const uint8_t* __restrict__ p0,
-                                             const uint8_t* __restrict__ p1, float fs, float ft) {
+// Bilinear colour between texels (i0, j0) and (i0 + 1, j0 + 1); value / 255.
+__device__ __forceinline__ float3 texel_lerp(const uint8_t* __restrict__ tex, int W, int H, int i0,
+                                             int j0, float fs, float ft) {
+    uint32_t lo0, hi0, lo1, hi1;
+    texel_square(tex, W, H, i0, j0, LoadTexels(), lo0, hi0, lo1, hi1);
     float2 r0, g0, b0, r1, g1, b1;
-    texel_pair(p0, r0, g0, b0);
-    texel_pair(p1, r1, g1, b1);
+    texel_channels(lo0, hi0, r0, g0, b0);
+    texel_channels(lo1, hi1, r1, g1, b1);
     constexpr float k = 1.0f / 255.0f;
     return make_float3(lerpf(lerpf(r0.x, r0.y, fs), lerpf(r1.x, r1.y, fs), ft) * k,
                        lerpf(lerpf(g0.x, g0.y, fs), lerpf(g1.x, g1.y, fs), ft) * k,
@@ -475,10 +476,10 @@ __device__ __forceinline__ float3 environment(const VolArgs& A, float3 d) {
     v = fminf(fmaxf(v, 0.0f), H - 1.0f);
     const int j0 = min(static_cast<int>(floorf(v)), A.bgH - 2);
     const float fv = v - static_cast<float>(j0);
+    if (i0 + 1 < A.bgW) return texel_lerp(A.bg, A.bgW, A.bgH, i0, j0, fu, fv);
+    // the pair that wraps: the last texel of a row and its first
     const uint8_t* r0 = A.bg + static_cast<size_t>(j0) * A.bgW * 3;
     const uint8_t* r1 = r0 + static_cast<size_t>(A.bgW) * 3;
-    if (i0 + 1 < A.bgW) return texel_lerp(r0 + 3 * i0, r1 + 3 * i0, fu, fv);
-    // the pair that wraps: the last texel of a row and its first
     float out[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -500,8 +501,7 @@ __device__ __forceinline__ float3 texel_bilinear(const uint8_t* tex, int W, int 
     const int i0 = min(static_cast<int>(floorf(s)), W - 2);
     const int j0 = min(static_cast<int>(floorf(t)), H - 2);
     const float fs = s - static_cast<float>(i0), ft = t - static_cast<float>(j0);
-    const uint8_t* r0 = tex + (static_cast<size_t>(j0) * W + i0) * 3;
-    return texel_lerp(r0, r0 + static_cast<size_t>(W) * 3, fs, ft);
+    return texel_lerp(tex, W, H, i0, j0, fs, ft);
 }
 
 // What the straight ray P + t d (t > 0) sees: the nearest textured plane it
