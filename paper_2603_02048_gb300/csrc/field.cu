@@ -110,8 +110,8 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
     }
     // this warp's row pair of nonzero words: lane l < 4 owns row l & 1, slice l >> 1
     unsigned* const nz_at =
-        H ? nz_bits + (static_cast<size_t>(2 * kk0 + (lane >> 1)) * (2 * row_pairs) + 2 * jj + (lane & 1)) *
-                          nz_words + word
+        H ? nz_bits + (static_cast<size_t>(2 * kk0 + (lane >> 1)) * (2 * row_pairs) + 2 * jj +
+                       (lane & 1)) * nz_words + word
           : nullptr;
     const size_t nz_step = static_cast<size_t>(4 * row_pairs) * nz_words;
     const int i = min(static_cast<int>(I), nx - 1);
@@ -145,7 +145,8 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
     // the multiplication by 1/2 commute), and walks two pairs at once: 256^3 FP16
     // build 183.7 against 181.5 us, 512^3 1564 against 1557
     float mx = 0.0f, my0 = 0.0f, my1 = 0.0f;
-    const float kx = MODE == 1 ? 1.0f : fx, ky0 = MODE == 1 ? 1.0f : fy0, ky1 = MODE == 1 ? 1.0f : fy1;
+    const float kx = MODE == 1 ? 1.0f : fx;
+    const float ky0 = MODE == 1 ? 1.0f : fy0, ky1 = MODE == 1 ? 1.0f : fy1;
 #pragma unroll(MODE == 1 ? 2 : 1)
     for (int kk = kk0; kk < kk1; ++kk) {
         const int K0 = 2 * kk - H, K1 = K0 + 1;  // grid slices of the pair
@@ -186,7 +187,9 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
             v11.gy = (od - (last_row ? oa : b0)) * ky1;
         }
         if (MODE == 1) {
-            auto peak = [](float m, float a, float b) { return fmaxf(m, fmaxf(fabsf(a), fabsf(b))); };
+            auto peak = [](float m, float a, float b) {
+                return fmaxf(m, fmaxf(fabsf(a), fabsf(b)));
+            };
             mn = peak(peak(mn, a0, a1), b0, b1);
             mx = peak(peak(mx, v00.gx, v10.gx), v01.gx, v11.gx);
             my0 = peak(my0, v00.gy, v01.gy);
@@ -234,7 +237,9 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
                 z11 = zero(w11);
                 uint2* to = static_cast<uint2*>(out) + o;
                 auto put = [&](int d) {
-                    if (valid) __stcs(reinterpret_cast<uint4*>(to + d), make_uint4(w00.x, w00.y, w01.x, w01.y));
+                    if (valid)
+                        __stcs(reinterpret_cast<uint4*>(to + d),
+                               make_uint4(w00.x, w00.y, w01.x, w01.y));
                     if (valid1)
                         __stcs(reinterpret_cast<uint4*>(to + static_cast<int>(row) + d),
                                make_uint4(w10.x, w10.y, w11.x, w11.y));
@@ -249,7 +254,8 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
             const unsigned n01 = __ballot_sync(0xffffffffu, valid && !z01);
             const unsigned n11 = __ballot_sync(0xffffffffu, valid1 && !z11);
             if (lane < 4 && static_cast<int>(jj) < row_pairs)
-                nz_at[(kk - kk0) * nz_step] = lane & 2 ? (lane & 1 ? n11 : n01) : (lane & 1 ? n10 : n00);
+                nz_at[(kk - kk0) * nz_step] =
+                    lane & 2 ? (lane & 1 ? n11 : n01) : (lane & 1 ? n10 : n00);
         }
         p0 = b0;
         p1 = b1;
@@ -280,10 +286,13 @@ __global__ void __launch_bounds__(256, field_blocks(MODE))
 }
 
 // A warp's stretch of the mask (1024 elements) with at least this many free
-// ones makes the volume sparse: the march then tests the mask at each sample.
-// Below it, over the whole volume, the test costs a load's latency and six
-// instructions a sample and saves next to nothing (720p view of a 192x160x224
-// turbulence volume without empty space: 194 us with it, 182 without).
+// ones makes the volume sparse: marches then ask the mask, RK4 at every sample,
+// Eq. 16 after a sample with dn = 0. In a volume without empty space the question
+// costs Eq. 16 little and RK4 a load's latency a sample, for nothing (720p views of
+// a 192x160x224 turbulence volume, asked and not: Eq. 16 at theta 1e-5 178 and 175
+// us, RK4 595 and 558, RK4 at half a voxel 1205 and 1070; a 64^3 128x128 RK4 view
+// 203 and 171). So the line is low, one stretch an eighth of which is free, and a
+// volume with a hole of that size only is marched as a sparse one.
 constexpr unsigned kSparseFree = 128;
 
 // The free-corner mask from the store pass's nonzero bits, a word (32
@@ -310,7 +319,8 @@ __global__ void __launch_bounds__(256)
     if (at < pair) {
         unsigned word = 0;
         for (unsigned done = 0; done < 32u && kk < pairs;) {
-            unsigned J = static_cast<unsigned>(__uint2float_rz(at) * per_row);  // at / row, off by one
+            // at / row, off by one at most
+            unsigned J = static_cast<unsigned>(__uint2float_rz(at) * per_row);
             if (J * row > at) --J;
             if ((J + 1u) * row <= at) ++J;
             const unsigned e = at - J * row, n = min(32u - done, min(row - e, pair - at));
@@ -386,8 +396,8 @@ __global__ void export_kernel(const void* __restrict__ data, int storage, unsign
 cudaError_t launch_field(const float* rho, int nx, int ny, int nz, float K, hh_volume_s* vol,
                          bool max_clear, cudaStream_t s) {
     // eight warps of 32 columns a block, rows padded to whole warps; blockIdx.y
-    // picks the run of slice pairs: eight, or fewer where that leaves the chip
-    // with less than four blocks an SM
+    // picks the run of slice pairs: eight, or fewer where that leaves the chip's
+    // 152 SMs with less than four blocks each
     const bool halo = vol->layout == HH_LAYOUT_ZPAIR;
     const dim3 block(256);
     auto grid_of = [&](int h, int& run) {
@@ -413,8 +423,9 @@ cudaError_t launch_field(const float* rho, int nx, int ny, int nz, float K, hh_v
         const dim3 max_grid = grid_of(0, max_run);
         launch_next(field_kernel<1, 0>, max_grid, block, s, rho, nx, ny, nz, K, max_run, 0, 0,
                     nullptr, nullptr, nullptr, vol->max_dev, vol->scales_dev);
-        launch_next(field_kernel<2, 1>, grid, block, s, rho, nx, ny, nz, K, run, vol->row, vol->pair,
-                    vol->data, vol->nz_dev, vol->sparse_dev, vol->max_dev, vol->scales_dev);
+        launch_next(field_kernel<2, 1>, grid, block, s, rho, nx, ny, nz, K, run, vol->row,
+                    vol->pair, vol->data, vol->nz_dev, vol->sparse_dev, vol->max_dev,
+                    vol->scales_dev);
         count_launch(2);
     }
     if (halo) {

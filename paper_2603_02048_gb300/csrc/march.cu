@@ -64,21 +64,21 @@ namespace {
 constexpr float kPi = 3.14159265358979323846f;
 
 // Resident 128-thread blocks per SM the single-view march kernels are compiled
-// for. Eq. 16: 8, i.e. at most 64 registers a thread (9 or 10 measured the same,
-// or slower where they spill). RK4: 6 (80 registers) on FP16, 5 (102) on FP32
-// storage, whose four samples a step otherwise spill (256^3 720p view 2514
-// against 2446 us, 64^3 128x128 164 against 140; FP16 1080p view 964 against 1014
-// with 5).
+// for. Eq. 16: 8, i.e. at most 64 registers a thread, at which FP32 storage spills
+// up to 28 bytes (9 or 10 blocks measured the same or slower). RK4: 6 (80
+// registers) on FP16; 5 (96, of which up to 8 bytes still spill) on FP32 storage,
+// whose four samples a step spill more at 6 (256^3 720p view 2514 against 2446 us,
+// 64^3 128x128 164 against 140; FP16 1080p view 964 against 1014 with 5).
 constexpr int march_blocks(int storage, int stepper) {
     return stepper != HH_STEP_RK4 ? 8 : storage == HH_STORE_FP32 ? 5 : 6;
 }
 // Resident 256-thread blocks per SM of the persistent batched kernel. More
-// warps hide more of the L2 latency as long as the step does not spill. Tile at
-// a time, FP16: 5 blocks (48 registers) against 4, 8 views of the 256^3 volume
-// 1085 against 1088 us (views in turn: 1148 against 1195), 32 views of the 512^3
-// one 9.34 against 9.77 ms. FP32, whose eight corners take twice the
-// registers: 4 blocks (64) against 3 and 5, 8 views 1171 against 1239 and 1367
-// us. RK4 and the refill state need more registers.
+// warps hide more of the L2 latency, until the step spills much of its state. Tile
+// at a time, FP16: 5 blocks (48 registers, 4 to 28 bytes spilled) against 4, 8
+// views of the 256^3 volume 1085 against 1088 us (views in turn: 1148 against
+// 1195), 32 views of the 512^3 one 9.34 against 9.77 ms. FP32, whose eight corners
+// take twice the registers: 4 blocks (64) against 3 and 5, 8 views 1171 against
+// 1239 and 1367 us. RK4 and the refill state need more registers.
 constexpr int batch_blocks(int storage, int stepper, bool refill) {
     if (stepper == HH_STEP_RK4 || refill) return 3;
     return storage == HH_STORE_FP32 ? 4 : 5;
@@ -257,7 +257,8 @@ __device__ __forceinline__ float div_approx(float a, float b) {
 int step_len(const hh_step_params& P) {
     const float least = 0x1p-100f;
     if (!P.adaptive) return P.h_fixed < least ? LEN_SUBNORMAL : LEN_FIXED;
-    const bool tiny = P.eps < 0x1p-39f || P.h_min < least || (P.theta_max > 0.0f && P.theta_max < least);
+    const bool tiny = P.eps < 0x1p-39f || P.h_min < least ||
+                      (P.theta_max > 0.0f && P.theta_max < least);
     return tiny ? LEN_SUBNORMAL : LEN_EQ18;
 }
 
@@ -265,12 +266,12 @@ int step_len(const hh_step_params& P) {
 // position + 1/2, the halo coordinate of the ZPAIR layout (the centre of
 // grid voxel i at u = i + 1; the march carries u, not the position):
 // i0 = floor(u), f = u - i0 (both from u itself: an index taken from the rounded
-// value would wait for it; march of the 256^3 frame 309 against 305 us). A position in [0, n] has u in [0.5, n + 0.5], so
-// both corners i0, i0 + 1 lie in the padded axis [0, n + 1], and the halo
-// copies make this the sample with the lattice coordinate clamped to the
-// voxel centres. The Euler march samples only accepted points, which lie in
-// the box (a NaN gives i0 = 0); CLAMP first clamps u to [0.5, n + 0.5] (NaN
-// to 0.5) for RK4 stage points, which may lie outside.
+// value would wait for it; march of the 256^3 frame 309 against 305 us). A
+// position in [0, n] has u in [0.5, n + 0.5], so both corners i0, i0 + 1 lie in
+// the padded axis [0, n + 1], and the halo copies make this the sample with the
+// lattice coordinate clamped to the voxel centres. The Euler march samples only
+// accepted points, which lie in the box (a NaN gives i0 = 0); CLAMP first clamps u
+// to [0.5, n + 0.5] (NaN to 0.5) for RK4 stage points, which may lie outside.
 template <bool CLAMP>
 __device__ __forceinline__ void axis_cell(float u, int n, int& i0, float& f) {
     if (CLAMP) u = fminf(fmaxf(u, 0.5f), static_cast<float>(n) + 0.5f);
@@ -356,16 +357,20 @@ __device__ __forceinline__ bool fetch_nonzero(const VolArgs& A, const void* __re
         // then y, then z with packed FP32x2 arithmetic, two channels per
         // instruction (measured 8 % faster there; on FP32 storage the 8-weight
         // form below is faster)
-        const uint2 r000 = __ldg(c00), r100 = __ldg(c00 + 2), r010 = __ldg(c10), r110 = __ldg(c10 + 2);
-        const uint2 r001 = __ldg(c01), r101 = __ldg(c01 + 2), r011 = __ldg(c11), r111 = __ldg(c11 + 2);
+        const uint2 r000 = __ldg(c00), r100 = __ldg(c00 + 2);
+        const uint2 r010 = __ldg(c10), r110 = __ldg(c10 + 2);
+        const uint2 r001 = __ldg(c01), r101 = __ldg(c01 + 2);
+        const uint2 r011 = __ldg(c11), r111 = __ldg(c11 + 2);
         const float2 tx = dup(fx), ty = dup(fy), tz = dup(fz);
         c = lerp4x2(lerp4x2(xlerp_fp16(r000, r100, tx), xlerp_fp16(r010, r110, tx), ty),
                     lerp4x2(xlerp_fp16(r001, r101, tx), xlerp_fp16(r011, r111, tx), ty), tz);
     } else {
         // the standard 8-corner weights (formed two at a time; the sum over
         // corners packed two channels at a time was slower, 317 against 308 us)
-        const float4 v000 = __ldg(c00), v100 = __ldg(c00 + 2), v010 = __ldg(c10), v110 = __ldg(c10 + 2);
-        const float4 v001 = __ldg(c01), v101 = __ldg(c01 + 2), v011 = __ldg(c11), v111 = __ldg(c11 + 2);
+        const float4 v000 = __ldg(c00), v100 = __ldg(c00 + 2);
+        const float4 v010 = __ldg(c10), v110 = __ldg(c10 + 2);
+        const float4 v001 = __ldg(c01), v101 = __ldg(c01 + 2);
+        const float4 v011 = __ldg(c11), v111 = __ldg(c11 + 2);
         const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
         const float2 y0 = make_float2(gy, fy), yz0 = mul2(y0, dup(gz)), yz1 = mul2(y0, dup(fz));
         const float2 w00 = mul2(dup(gx), yz0), w10 = mul2(dup(fx), yz0);  // [x][z], over y
@@ -619,8 +624,8 @@ template <int STORAGE, int LEN, int ADDR, bool MASK, bool CLAMP>
 __device__ __forceinline__ float3 perp_rate(const VolArgs& A, const void* __restrict__ vol,
                                             float3 u, float3 w, float s_n, float s_g, float& n,
                                             float& gperp_norm, uint32_t& flags) {
-    return perp_of<STORAGE, LEN>(fetch<STORAGE, ADDR, MASK, CLAMP>(A, vol, u, flags), w, s_n, s_g, n,
-                                 gperp_norm);
+    return perp_of<STORAGE, LEN>(fetch<STORAGE, ADDR, MASK, CLAMP>(A, vol, u, flags), w, s_n, s_g,
+                                 n, gperp_norm);
 }
 
 // Per-ray state of the march: primary direction w_ref, deflection d, biased
@@ -696,24 +701,25 @@ __device__ __forceinline__ bool ray_step(const VolArgs& V, const void* __restric
     if (STEPPER == HH_STEP_RK4) {
         float n1, gpn, n2, n3, n4, unused;
         const float3 w1 = wr + d;
-        const float3 gp1 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, C, w1, R.sn, R.sg, n1, gpn, R.flags);
+        const float3 gp1 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, C, w1, R.sn, R.sg, n1,
+                                                                     gpn, R.flags);
         ds = step_length<LEN>(V, n1, gpn);
         const float hds = 0.5f * ds;
         const float3 k1 = (div_approx<LEN>(1.0f, n1) * gsc) * gp1;
         const float3 d2 = fma3(hds, k1, d);
         const float3 w2 = wr + d2;
-        const float3 gp2 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, fma3(hds, w1, C), w2, R.sn, R.sg, n2,
-                                                    unused, R.flags);
+        const float3 gp2 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(
+            V, vol, fma3(hds, w1, C), w2, R.sn, R.sg, n2, unused, R.flags);
         const float3 k2 = (div_approx<LEN>(1.0f, n2) * gsc) * gp2;
         const float3 d3 = fma3(hds, k2, d);
         const float3 w3 = wr + d3;
-        const float3 gp3 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, fma3(hds, w2, C), w3, R.sn, R.sg, n3,
-                                                    unused, R.flags);
+        const float3 gp3 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(
+            V, vol, fma3(hds, w2, C), w3, R.sn, R.sg, n3, unused, R.flags);
         const float3 k3 = (div_approx<LEN>(1.0f, n3) * gsc) * gp3;
         const float3 d4 = fma3(ds, k3, d);
         const float3 w4 = wr + d4;
-        const float3 gp4 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(V, vol, fma3(ds, w3, C), w4, R.sn, R.sg, n4,
-                                                    unused, R.flags);
+        const float3 gp4 = perp_rate<STORAGE, LEN, ADDR, MASK, true>(
+            V, vol, fma3(ds, w3, C), w4, R.sn, R.sg, n4, unused, R.flags);
         const float3 k4 = (div_approx<LEN>(1.0f, n4) * gsc) * gp4;
         // k1 + 2 (k2 + k3) + k4 (every k is a product: the adds are kept
         // unfused, __fadd_rn, so no product is folded into them)
@@ -1076,9 +1082,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // What a warp of the serving worker keeps between tiles, in shared memory: the
-// view record of its current tile and its job. In registers the march's loop
-// spilled (six requests of three views on a 384^3 FP16 volume: 12.2 against 11.4
-// ms).
+// view record of its current tile and its job. In registers they made the
+// march's loop spill more (six requests of three views on a 384^3 FP16 volume, four
+// blocks: 12.2 against 11.4 ms).
 struct alignas(16) WorkerWarp {
     ViewArgs view;
     unsigned long long vol, scales;  // addresses of the job's volume and its FP16 scales
@@ -1092,7 +1098,7 @@ struct alignas(16) WorkerWarp {
 
 // Resident 256-thread blocks per SM of the serving worker: as the batched
 // kernel's (FP16: 5 against 4, six requests of three views on a 384^3 volume in
-// 10.65 against 11.4 ms).
+// 10.65 against 11.4 ms, although 60 to 68 bytes spill at 5).
 constexpr int worker_blocks(int storage, int stepper) {
     return batch_blocks(storage, stepper, false);
 }
@@ -1225,7 +1231,8 @@ __global__ void __launch_bounds__(256, worker_blocks(STORAGE, STEPPER))
             __syncwarp();
             const unsigned* src = reinterpret_cast<const unsigned*>(
                 views + static_cast<size_t>(S.view_begin + lo) * sizeof(ViewArgs));
-            for (int w = lane; w < kWords; w += 32) reinterpret_cast<unsigned*>(&C)[w] = __ldcg(src + w);
+            for (int w = lane; w < kWords; w += 32)
+                reinterpret_cast<unsigned*>(&C)[w] = __ldcg(src + w);
             __syncwarp();
             if (lane == 0) {
                 S.view_first = C.tile_begin;
@@ -1360,8 +1367,9 @@ struct WorkerLaunch {
 template <int ST, int SP, int LEN>
 struct WorkerOccupancy {
     static void run(bool any, int threads, int* blocks_per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, worker_kernel<ST, SP, LEN>(any),
-                                                      threads, (threads / 32) * sizeof(WorkerWarp));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            blocks_per_sm, worker_kernel<ST, SP, LEN>(any), threads,
+            (threads / 32) * sizeof(WorkerWarp));
     }
 };
 

@@ -72,8 +72,9 @@ __device__ __forceinline__ void footprint(float x, float reach, int n, int& lo, 
 // Clears n floats, sixteen a thread in 16-byte stores, and the two words at
 // max_bits (nullable). A kernel and not a memset so that the splat's blocks can
 // start, and read their particles, behind it (launch_next): the density of
-// 262,144 particles on 256^3 103.3 against 99.1 us. What bounds it: L2 writes. It is launched as an ordinary kernel: the particles are complete
-// before it starts, so the splat may read them before it ends.
+// 262,144 particles on 256^3 103.3 against 99.1 us. What bounds it: L2 writes. It
+// is launched as an ordinary kernel: the particles are complete before it starts,
+// so the splat may read them before it ends.
 __global__ void __launch_bounds__(256) zero_kernel(float* __restrict__ p, size_t n,
                                                    unsigned* __restrict__ max_bits) {
     release_next();
@@ -190,11 +191,12 @@ __device__ __forceinline__ float dist_or_inf(int k, int n, float x) {
 // the M4 is evaluated as m norm (2 t^3 - u^3), t = 1 - r / 2h, u = sat(1 - r / h),
 // equal to its two pieces on [0, 2h); else by pieces (m4_mass), as fast and
 // without the rounding of 1 / h in every distance.
-// What bounds it: the L2 reductions (0.7-0.8 T float additions a second) and
-// the issue rate, together at N = 8 (83 % issue, 262,144 particles on 256^3 in
-// 90 us). Packed FP32x2 arithmetic issues fewer instructions but is no faster;
-// vector reductions (.v2, .v4 on aligned x runs, or on a bricked density) are
-// slower there (111-184 us). 60,011 particles on 161x118x97, with the
+// What bounds it is the reductions' way to L2 or the issue rate, near each other:
+// at N = 8 83 % issue and 31 M sector reductions in 90 us (262,144 particles on
+// 256^3), 0.78 T float additions a second at N = 12. Neither's own ceiling is
+// measured; 6 to 7 % fewer instructions took the same time, packed FP32x2
+// arithmetic, which issues fewer too, as well. Vector reductions (.v2, .v4 on
+// aligned x runs, or on a bricked density) are slower there (111-184 us). 60,011 particles on 161x118x97, with the
 // density's memset, against splat_warp_kernel (N <= 8: against the 8-slot box):
 //   h     1 (N = 4)  1.5 (6)  2.5 (10)  3 (12)  4 (16)
 //   before   27        27        87       137     228 us
@@ -434,7 +436,8 @@ cudaError_t launch_splat(const float4* xyzm, int64_t n, int nx, int ny, int nz, 
     int e2 = 0;
     const bool unit = hd < 0.5 || std::frexp(hd, &e2) == 0.5;
     auto box = [&](auto kernel, int lanes) {
-        launch_next(kernel, blocks(32 / lanes), threads, s, xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
+        launch_next(kernel, blocks(32 / lanes), threads, s, xyzm, n, nx, ny, nz, h, inv_h, norm,
+                    rho);
     };
     // the smallest box that holds the support (4h slots an axis)
     if (hd <= 1.0)
@@ -450,7 +453,8 @@ cudaError_t launch_splat(const float4* xyzm, int64_t n, int nx, int ny, int nz, 
     else if (hd <= 4.0)
         box(splat_box_kernel<16, 16, false>, 16);
     else
-        launch_next(splat_warp_kernel<kParticlesPerWarp>, blocks(kParticlesPerWarp), threads, s, xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
+        launch_next(splat_warp_kernel<kParticlesPerWarp>, blocks(kParticlesPerWarp), threads, s,
+                    xyzm, n, nx, ny, nz, h, inv_h, norm, rho);
     count_launch();
     return cudaGetLastError();
 }
