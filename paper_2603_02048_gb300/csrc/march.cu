@@ -439,7 +439,7 @@ __device__ __forceinline__ float3 renormalize(float3 w1, float3 d1) {
 
 struct LoadTexels {
     __device__ __forceinline__ uint32_t operator()(const uint8_t* p) const { return __ldg(p); }
-    __device__ __forceinline__ uint32_t operator()(const uint32_t* p) const { return __ldg(p); }
+    __device__ __forceinline__ uint32_t operator()(const uint16_t* p) const { return __ldg(p); }
 };
 
 // Channels of a pair of texels read as lo, hi.
@@ -451,10 +451,10 @@ __device__ __forceinline__ void texel_channels(uint32_t lo, uint32_t hi, float2&
 }
 
 // Bilinear colour between texels (i0, j0) and (i0 + 1, j0 + 1); value / 255.
-__device__ __forceinline__ float3 texel_lerp(const uint8_t* __restrict__ tex, int W, int H, int i0,
-                                             int j0, float fs, float ft) {
+__device__ __forceinline__ float3 texel_lerp(const uint8_t* __restrict__ tex, int W, int i0, int j0,
+                                             float fs, float ft) {
     uint32_t lo0, hi0, lo1, hi1;
-    texel_square(tex, W, H, i0, j0, LoadTexels(), lo0, hi0, lo1, hi1);
+    texel_square(tex, W, i0, j0, LoadTexels(), lo0, hi0, lo1, hi1);
     float2 r0, g0, b0, r1, g1, b1;
     texel_channels(lo0, hi0, r0, g0, b0);
     texel_channels(lo1, hi1, r1, g1, b1);
@@ -481,7 +481,7 @@ __device__ __forceinline__ float3 environment(const VolArgs& A, float3 d) {
     v = fminf(fmaxf(v, 0.0f), H - 1.0f);
     const int j0 = min(static_cast<int>(floorf(v)), A.bgH - 2);
     const float fv = v - static_cast<float>(j0);
-    if (i0 + 1 < A.bgW) return texel_lerp(A.bg, A.bgW, A.bgH, i0, j0, fu, fv);
+    if (i0 + 1 < A.bgW) return texel_lerp(A.bg, A.bgW, i0, j0, fu, fv);
     // the pair that wraps: the last texel of a row and its first
     const uint8_t* r0 = A.bg + static_cast<size_t>(j0) * A.bgW * 3;
     const uint8_t* r1 = r0 + static_cast<size_t>(A.bgW) * 3;
@@ -506,7 +506,7 @@ __device__ __forceinline__ float3 texel_bilinear(const uint8_t* tex, int W, int 
     const int i0 = min(static_cast<int>(floorf(s)), W - 2);
     const int j0 = min(static_cast<int>(floorf(t)), H - 2);
     const float fs = s - static_cast<float>(i0), ft = t - static_cast<float>(j0);
-    return texel_lerp(tex, W, H, i0, j0, fs, ft);
+    return texel_lerp(tex, W, i0, j0, fs, ft);
 }
 
 // What the straight ray P + t d (t > 0) sees: the nearest textured plane it

@@ -20,6 +20,13 @@ struct Load {
         check(p, 1);
         return *p;
     }
+    uint32_t operator()(const uint16_t* p) const {
+        check(p, 2);
+        if (reinterpret_cast<uintptr_t>(p) % 2) ++g_outside;  // misaligned
+        uint16_t v;
+        std::memcpy(&v, p, 2);
+        return v;
+    }
     uint32_t operator()(const uint32_t* p) const {
         check(p, 4);
         uint32_t v;
@@ -41,7 +48,7 @@ int main() {
                     for (int i = 0; i <= W - 2; ++i) {
                         uint32_t w[2][2];
                         g_outside = 0;
-                        hh::texel_square(tex, W, H, i, j, Load(), w[0][0], w[0][1], w[1][0], w[1][1]);
+                        hh::texel_square(tex, W, i, j, Load(), w[0][0], w[0][1], w[1][0], w[1][1]);
                         bool ok = g_outside == 0;
                         for (int r = 0; r < 2; ++r)
                             for (int b = 0; b < 6; ++b)
